@@ -114,7 +114,10 @@ int rosetta_params_init(rosetta_ctx **out, const rosetta_params *p, int cuda_dev
  * four-prime kernel's (on a 228 KB SM at N = 4096, l = 2: all n but 10752 to
  * 12799; at N = 8192, l = 3: n <= 15871); e.g. N = 4096, l = 2, beta = 15
  * and N = 8192, l = 3, beta = 14.  Either way the outputs are the same words: the product is
- * exact.  Fixed at rosetta_params_init.  Returns 3 or 4, or INVALID_ARG for a
+ * exact.  (At N = 2048 with one level and beta <= 24 a context that reports 4
+ * runs the parts of a batch that fill the GPU over three of them and places
+ * the missing multiple of their product with a bounded-error float estimate:
+ * the same words again.)  Fixed at rosetta_params_init.  Returns 3 or 4, or INVALID_ARG for a
  * NULL context. */
 int rosetta_ntt_primes(const rosetta_ctx *ctx);
 

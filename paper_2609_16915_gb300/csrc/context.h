@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "rosetta.h"
 #include "internal.h"
 
@@ -12,6 +14,7 @@ struct rosetta_ctx {
   rosetta_params prm{};
   int device = 0;
   uint32_t logN = 0;
+  uint32_t sms = 1;               // SMs of the device
   bool dig16 = false;
   rosetta::CrtConsts cc{};
   uint2 *d_tw = nullptr;          // [kPrimes][N]
@@ -20,6 +23,15 @@ struct rosetta_ctx {
   uint32_t br_primes = rosetta::kPrimes;
   uint2 *d_tw31 = nullptr;        // [kPrimes31][N], or null
   rosetta::CrtConsts cc31{};
+  // the worker-per-ciphertext kernel of the standard ring (three 28-bit primes
+  // and the float quotient), beside the cluster kernel's tables and key: the
+  // primes' twiddles and the pass table [4][N], the key transform's table
+  bool br_qf = false;
+  uint2 *d_tw_qf = nullptr;
+  std::vector<uint2> tw_qf_host;
+  double2 *d_tw_f64 = nullptr;    // [N/2]
+  rosetta::CrtConsts cc_qf{};
+  uint32_t *d_bsk_qf = nullptr;   // [n][4][2][2][N]
   uint32_t *d_bsk = nullptr;      // transform domain over br_primes primes
   size_t bsk_words = 0;           // its size in 32-bit words
   uint64_t *d_ksk = nullptr;      // raw [kN][l_ks][n+1]
@@ -66,3 +78,15 @@ inline void br_key_args(const rosetta_ctx *c, rosetta::BrArgs *a) {
   a->tw = three ? c->d_tw31 : c->d_tw;
   a->cc = three ? c->cc31 : c->cc;
 }
+
+// The same for the worker-per-ciphertext kernel.
+inline void br_solo_key_args(const rosetta_ctx *c, rosetta::BrArgs *a) {
+  a->bsk = c->d_bsk_qf;
+  a->primes = rosetta::kPrimes;
+  a->tw = c->d_tw_qf;
+  a->cc = c->cc_qf;
+}
+
+// Blind rotation of a.batch ciphertexts (a: br_key_args filled in) on the
+// kernels that suit the batch.
+cudaError_t run_blind_rotate(const rosetta_ctx *c, const rosetta::BrArgs &a, cudaStream_t s);

@@ -22,6 +22,14 @@ constexpr uint32_t kPrimeList[kPrimes] = {268369921u, 268271617u, 268238849u, 26
 constexpr int kPrimes31 = 3;
 constexpr uint32_t kPrime31List[kPrimes31] = {2147352577u, 2147205121u, 2147074049u};
 
+// The float quotient (QF): a blind rotation over the first three 28-bit primes
+// whose fourth CTA estimates the product's size X / M3 with single-precision
+// complex transforms (cfft.cuh) instead of computing a fourth residue.  The
+// estimate arrives scaled by 2^kQfShift; |X| / M3 <= 2^(kQfBits - 83.99).
+constexpr int kPrimesQf = 3;
+constexpr int kQfShift = 16;
+constexpr int kQfBits = 98;
+
 struct PrimeConsts {
   uint32_t p;
   uint32_t p_inv;     // p^{-1} mod 2^32 (Montgomery reduction)
@@ -35,6 +43,7 @@ struct PrimeConsts {
 struct CrtConsts {
   PrimeConsts pr[kPrimes];
   uint64_t M_mod64;   // M mod 2^64
+  uint64_t qf_base;   // 2^(31 - kQfShift) M mod 2^64: undoes the offset of crt_quotient_qf
 };
 
 struct BrArgs {
@@ -99,11 +108,21 @@ inline cudaClusterSchedulingPolicy br_cluster_policy(K kern, int threads, size_t
 }
 
 // host-side tables (tables.cu): twiddles and CRT constants of the 28-bit set
-// (primes = kPrimes) or of the 31-bit set (primes = kPrimes31)
-bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host /*[primes][N]*/, CrtConsts *cc);
+// (primes = kPrimes; the first `use` of them) or of the 31-bit set (primes =
+// kPrimes31); tw_host may be null
+bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host /*[use][N]*/, CrtConsts *cc, uint32_t use = 0);
+// twiddles of the float transforms of N/2 complex values: the pass table the
+// kernels read (float4 entries, at most N uint2 words) and the whole double
+// table [N/2] of the key transform
+void build_cfft_tables(uint32_t logN, float4 *pass_tw, double2 *tw);
 
 // launchers; return cudaSuccess or the launch error
 size_t br_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, bool dig16);
+// one worker per ciphertext, float quotient (blind_rotate_solo.cu): a.bsk, a.tw,
+// a.cc of the float-quotient set, tw_host the host copy of its tables, `workers` (1 .. 3) ciphertexts per CTA
+bool br_solo_supported(uint32_t logN, uint32_t level, uint32_t base_log);
+size_t br_solo_smem_bytes(uint32_t n, uint32_t workers);
+cudaError_t launch_blind_rotate_solo(const BrArgs &a, const uint2 *tw_host, uint32_t workers, cudaStream_t s);
 // a.primes selects the kernel: the four-prime one or the three-prime one
 cudaError_t launch_blind_rotate(const BrArgs &a, uint32_t logN, bool dig16, cudaStream_t s);
 // three-prime kernel (blind_rotate3.cu): 16-bit digits, compiled ring sizes and levels only
@@ -112,6 +131,10 @@ size_t br3_smem_bytes(uint32_t logN, uint32_t level, uint32_t n);
 cudaError_t launch_blind_rotate3(const BrArgs &a, uint32_t logN, cudaStream_t s);
 cudaError_t launch_bsk_transform(const uint64_t *raw, uint32_t *out, const uint2 *tw, const CrtConsts &cc,
                                  uint32_t logN, uint32_t n, uint32_t level, uint32_t primes, cudaStream_t s);
+// the key of a blind rotation with the float quotient: three primes' blocks
+// and the float transforms' in the fourth's place (tw: the primes', tw_f64: [N/2])
+cudaError_t launch_bsk_transform_qf(const uint64_t *raw, uint32_t *out, const uint2 *tw, const double2 *tw_f64,
+                                    const CrtConsts &cc, uint32_t logN, uint32_t n, uint32_t level, cudaStream_t s);
 cudaError_t launch_keyswitch(const KsArgs &a, cudaStream_t s);
 // transform `count` raw keys [count][rows][2][N] to [count][prime][rows][2][N]
 // over the 28-bit set (primes = kPrimes) or the 31-bit set (kPrimes31)

@@ -8,6 +8,8 @@
 #pragma once
 #include <stdint.h>
 
+#include "internal.h"
+
 namespace rosetta {
 
 // Shoup multiplication by a constant w < p with companion ws = floor(w 2^32 / p):
@@ -42,6 +44,27 @@ __device__ __forceinline__ uint32_t crt_quotient(uint32_t ysum) { return (ysum +
 // Only parameter sets whose exact integer value X obeys |X| <= 0.45 M take
 // this prime set, so the estimate stays within 0.46 of the integer.
 __device__ __forceinline__ uint32_t crt_quotient31(uint32_t ysum) { return (ysum + (1u << 27)) >> 28; }
+
+// The quotient of three 28-bit primes where X may be many times their product
+// M3: round(sum_q y_q / p_q - X / M3), from ysum = sum_q (y_q >> 17) and est =
+// 2^kQfShift X / M3 as the float transforms give it, plus an offset of
+// 2^(31 - kQfShift) that keeps it positive.  The primes lie in (2^28 - 2^18,
+// 2^28): y / 2^28 undershoots y / p by less than 2^-7 per prime (the shift adds
+// 2^-11), the three together by less than 2^-5.  est is within
+// 100 x 2^-24 x 2^98 / 2^83.99 < 0.1 of its exact value (cfft.cuh; |X| <=
+// 2^98), so the sum stays within 0.14 of an integer and rounds to it; |est|
+// <= 2^30.02 fits the conversion.
+__device__ __forceinline__ uint32_t qf_quotient(uint32_t ysum, float est) {
+  static_assert(kQfShift > 11, "ysum counts units of 2^-11");
+  return ((ysum << (kQfShift - 11)) + (1u << 31) + (1u << (kQfShift - 1)) -
+          static_cast<uint32_t>(__float2int_rn(est))) >> kQfShift;
+}
+
+// y0 >> 17 in the low and y1 >> 17 in the high half (y < 2^31: three such words
+// add without a carry between the halves).
+__device__ __forceinline__ uint32_t qf_pack(uint32_t y0, uint32_t y1) {
+  return (__byte_perm(y0, y1, 0x7632) >> 1) & 0x7FFF7FFFu;
+}
 
 // x in [0, 2b) -> [0, b) for a bound b: one subtraction when x >= b.
 __device__ __forceinline__ uint32_t cond_sub(uint32_t x, uint32_t b) {

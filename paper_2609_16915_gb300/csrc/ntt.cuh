@@ -33,7 +33,7 @@ __host__ __device__ constexpr int ilog2(int x) { return x <= 1 ? 0 : 1 + ilog2(x
 
 template <int LOGN, int E = 8>
 struct NttShape {
-  static_assert(E == 8 || E == 16, "8 or 16 values per thread");
+  static_assert(E == 4 || E == 8 || E == 16, "4, 8 or 16 values per thread");
   static constexpr int N = 1 << LOGN;
   static constexpr int T = N / E;                    // threads per transform
   static constexpr int RAD = ilog2(E);               // stages per full pass
@@ -136,10 +136,18 @@ __host__ __device__ constexpr bool inv_corrects(int q) {
   }
 }
 
+// The transforms read the twiddles of stage S, entries [2^S, 2^(S+1)), through
+// tw_at and load_twiddles, so that a kernel can hold them in its own way; by
+// default the table is one shared-memory array.
+template <int S>
+__device__ __forceinline__ uint2 tw_at(const uint2 *tw, uint32_t idx) {
+  return tw[idx];
+}
+
 // Load CNT (a power of two) consecutive twiddle pairs starting at an index
 // that is a multiple of CNT: one 8-byte or CNT/2 16-byte shared loads.
-template <int CNT>
-__device__ __forceinline__ void load_twiddles(const uint2 *__restrict__ tw, uint32_t start, uint2 (&w)[CNT]) {
+template <int S, int CNT>
+__device__ __forceinline__ void load_twiddles(const uint2 *tw, uint32_t start, uint2 (&w)[CNT]) {
   if constexpr (CNT == 1) {
     w[0] = tw[start];
   } else {
@@ -153,8 +161,8 @@ __device__ __forceinline__ void load_twiddles(const uint2 *__restrict__ tw, uint
   }
 }
 
-template <int LOGN, int E, int NP, int S0, int H, int U, bool P31>
-__device__ __forceinline__ void fwd_stage(uint32_t (&x)[NP][E], const uint2 *__restrict__ tw, uint32_t tau,
+template <int LOGN, int E, int NP, int S0, int H, int U, bool P31, class TW>
+__device__ __forceinline__ void fwd_stage(uint32_t (&x)[NP][E], const TW &tw, uint32_t tau,
                                           uint32_t p, uint32_t two_p, uint32_t eight_p) {
   constexpr uint32_t N = 1u << LOGN;
   constexpr uint32_t SIG = N >> (S0 + H);
@@ -166,7 +174,7 @@ __device__ __forceinline__ void fwd_stage(uint32_t (&x)[NP][E], const uint2 *__r
     // last pass: the thread's groups are consecutive, so are their twiddles
     constexpr int CNT = NB << U;
     uint2 w[CNT];
-    load_twiddles<CNT>(tw, (1u << S) + tau * CNT, w);
+    load_twiddles<S>(tw, (1u << S) + tau * CNT, w);
 #pragma unroll
     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -188,7 +196,7 @@ __device__ __forceinline__ void fwd_stage(uint32_t (&x)[NP][E], const uint2 *__r
 #pragma unroll
       for (int q = 0; q < (1 << H); ++q) {
         if (q & HALF) continue;
-        const uint2 w = tw[(1u << S) + (g << U) + (q >> (H - U))];
+        const uint2 w = tw_at<S>(tw, (1u << S) + (g << U) + (q >> (H - U)));
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
           if constexpr (P31)
@@ -201,8 +209,8 @@ __device__ __forceinline__ void fwd_stage(uint32_t (&x)[NP][E], const uint2 *__r
   }
 }
 
-template <int LOGN, int E, int NP, int S0, int H, int U, bool P31>
-__device__ __forceinline__ void inv_stage(uint32_t (&x)[NP][E], const uint2 *__restrict__ tw, uint32_t tau,
+template <int LOGN, int E, int NP, int S0, int H, int U, bool P31, class TW>
+__device__ __forceinline__ void inv_stage(uint32_t (&x)[NP][E], const TW &tw, uint32_t tau,
                                           uint32_t p, uint32_t eight_p) {
   constexpr bool LAST = (S0 + H == LOGN);  // the pass the inverse starts with
   constexpr uint32_t N = 1u << LOGN;
@@ -215,7 +223,7 @@ __device__ __forceinline__ void inv_stage(uint32_t (&x)[NP][E], const uint2 *__r
     // W[2^{s+1}-1-G], which starts at 2^{s+1} - (tau+1)*CNT
     constexpr int CNT = NB << U;
     uint2 w[CNT];
-    load_twiddles<CNT>(tw, (2u << S) - (tau + 1) * CNT, w);
+    load_twiddles<S>(tw, (2u << S) - (tau + 1) * CNT, w);
 #pragma unroll
     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -239,7 +247,7 @@ __device__ __forceinline__ void inv_stage(uint32_t (&x)[NP][E], const uint2 *__r
       for (int q = 0; q < (1 << H); ++q) {
         if (q & HALF) continue;
         const uint32_t G = (g << U) + (q >> (H - U));
-        const uint2 w = tw[(2u << S) - 1u - G];
+        const uint2 w = tw_at<S>(tw, (2u << S) - 1u - G);
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
           if constexpr (P31)
@@ -253,15 +261,15 @@ __device__ __forceinline__ void inv_stage(uint32_t (&x)[NP][E], const uint2 *__r
   }
 }
 
-template <int LOGN, int E, int NP, int S0, int H, bool P31, int U = 0>
-__device__ __forceinline__ void fwd_pass(uint32_t (&x)[NP][E], const uint2 *tw, uint32_t tau, uint32_t p,
+template <int LOGN, int E, int NP, int S0, int H, bool P31, int U = 0, class TW>
+__device__ __forceinline__ void fwd_pass(uint32_t (&x)[NP][E], const TW &tw, uint32_t tau, uint32_t p,
                                          uint32_t two_p, uint32_t eight_p) {
   fwd_stage<LOGN, E, NP, S0, H, U, P31>(x, tw, tau, p, two_p, eight_p);
   if constexpr (U + 1 < H) fwd_pass<LOGN, E, NP, S0, H, P31, U + 1>(x, tw, tau, p, two_p, eight_p);
 }
 
-template <int LOGN, int E, int NP, int S0, int H, bool P31, int U = H - 1>
-__device__ __forceinline__ void inv_pass(uint32_t (&x)[NP][E], const uint2 *tw, uint32_t tau, uint32_t p,
+template <int LOGN, int E, int NP, int S0, int H, bool P31, int U = H - 1, class TW>
+__device__ __forceinline__ void inv_pass(uint32_t (&x)[NP][E], const TW &tw, uint32_t tau, uint32_t p,
                                          uint32_t eight_p) {
   inv_stage<LOGN, E, NP, S0, H, U, P31>(x, tw, tau, p, eight_p);
   if constexpr (U > 0) inv_pass<LOGN, E, NP, S0, H, P31, U - 1>(x, tw, tau, p, eight_p);
@@ -277,10 +285,23 @@ __host__ __device__ constexpr int pass_group_warps() {
   return (1 << (LOGN - S0)) <= 32 * E ? 1 : (1 << (LOGN - S0)) / (32 * E);
 }
 
-template <int G, int WARPS>
-__device__ __forceinline__ void group_sync(uint32_t tau) {
+// The threads of a transform: a whole CTA, or (several transforms per CTA) one
+// group of `threads` threads with hardware barrier `id`.
+struct CtaThreads {
+  static constexpr bool kWhole = true, kPairs = false;
+};
+struct GroupThreads {
+  static constexpr bool kWhole = false, kPairs = true;  // two polynomials cross the exchange buffer as pairs of words
+  uint32_t id, threads;
+  __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+};
+
+template <int G, int WARPS, class TH>
+__device__ __forceinline__ void group_sync(uint32_t tau, const TH &th) {
   if constexpr (G <= 1) {
     __syncwarp();
+  } else if constexpr (!TH::kWhole) {
+    th.sync();
   } else if constexpr (G >= WARPS) {
     __syncthreads();
   } else {
@@ -346,29 +367,91 @@ __device__ __forceinline__ void xb_load(const uint32_t *buf, uint32_t (&v)[E], u
   }
 }
 
+// The same for two polynomials whose words travel side by side (8-byte
+// elements, half the accesses): 2 pad elements after every 16 keep every pass
+// free of bank conflicts (half-warps of 8-byte accesses, quarter-warps of the
+// last pass's 16-byte ones), and again the padding of base and offset adds.
+__host__ __device__ constexpr uint32_t xb_pad2(uint32_t i) { return i + ((i >> 4) << 1); }
+
+template <int LOGN, int E, int S0, int H>
+__device__ __forceinline__ uint32_t xb2_base(uint32_t tau) {
+  constexpr uint32_t N = 1u << LOGN, SIG = N >> (S0 + H), SPAN = N >> S0;
+  if constexpr (SIG == 1) {
+    return xb_pad2(E * tau);
+  } else {
+    static_assert((1 << H) == E && SIG % 4 == 0 && (SIG >= 16 || SIG == 4), "padding that adds");
+    return xb_pad2((tau / SIG) * SPAN + tau % SIG);
+  }
+}
+
+template <int LOGN, int E, int S0, int H>
+__device__ __forceinline__ void xb2_store(uint2 *buf, const uint32_t (&v)[2][E], uint32_t tau) {
+  uint2 *b = buf + xb2_base<LOGN, E, S0, H>(tau);
+  if constexpr (S0 + H == LOGN) {
+    uint4 *p = reinterpret_cast<uint4 *>(b);
+#pragma unroll
+    for (int k = 0; k < E / 2; ++k) p[k] = make_uint4(v[0][2 * k], v[1][2 * k], v[0][2 * k + 1], v[1][2 * k + 1]);
+  } else {
+    constexpr uint32_t SIG = (1u << LOGN) >> (S0 + H);
+#pragma unroll
+    for (int e = 0; e < E; ++e) b[xb_pad2(e * SIG)] = make_uint2(v[0][e], v[1][e]);
+  }
+}
+
+template <int LOGN, int E, int S0, int H>
+__device__ __forceinline__ void xb2_load(const uint2 *buf, uint32_t (&v)[2][E], uint32_t tau) {
+  const uint2 *b = buf + xb2_base<LOGN, E, S0, H>(tau);
+  if constexpr (S0 + H == LOGN) {
+    const uint4 *p = reinterpret_cast<const uint4 *>(b);
+#pragma unroll
+    for (int k = 0; k < E / 2; ++k) {
+      const uint4 a = p[k];
+      v[0][2 * k] = a.x;
+      v[1][2 * k] = a.y;
+      v[0][2 * k + 1] = a.z;
+      v[1][2 * k + 1] = a.w;
+    }
+  } else {
+    constexpr uint32_t SIG = (1u << LOGN) >> (S0 + H);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const uint2 a = b[xb_pad2(e * SIG)];
+      v[0][e] = a.x;
+      v[1][e] = a.y;
+    }
+  }
+}
+
 // Move NP register sets from the layout of pass A to that of pass B through
 // the exchange buffer xb (XBUF polynomials of NttShape::XB_WORDS words each).
 // The leading barrier protects xb from readers of the previous exchange; both
 // barriers cover only the warps whose data the exchange mixes.
-template <int LOGN, int E, int NP, int XBUF, int S0A, int HA, int S0B, int HB>
-__device__ __forceinline__ void exchange(uint32_t (&x)[NP][E], uint32_t *xb, uint32_t tau) {
+template <int LOGN, int E, int NP, int XBUF, int S0A, int HA, int S0B, int HB, class TH = CtaThreads>
+__device__ __forceinline__ void exchange(uint32_t (&x)[NP][E], uint32_t *xb, uint32_t tau, const TH &th = TH()) {
   constexpr int W = NttShape<LOGN, E>::XB_WORDS;
   constexpr int G = pass_group_warps<LOGN, E, (S0A < S0B ? S0A : S0B)>();
   constexpr int WARPS = NttShape<LOGN, E>::T / 32 > 0 ? NttShape<LOGN, E>::T / 32 : 1;
   static_assert(XBUF == 1 || XBUF == NP, "exchange buffer must hold one or all polynomials");
-  if constexpr (XBUF == NP) {
-    group_sync<G, WARPS>(tau);
+  if constexpr (TH::kPairs) {
+    static_assert(NP == 2 && XBUF == 2, "pairs of two polynomials");
+    uint2 *xb2 = reinterpret_cast<uint2 *>(xb);
+    group_sync<G, WARPS>(tau, th);
+    xb2_store<LOGN, E, S0A, HA>(xb2, x, tau);
+    group_sync<G, WARPS>(tau, th);
+    xb2_load<LOGN, E, S0B, HB>(xb2, x, tau);
+  } else if constexpr (XBUF == NP) {
+    group_sync<G, WARPS>(tau, th);
 #pragma unroll
     for (int k = 0; k < NP; ++k) xb_store<LOGN, E, S0A, HA>(xb + k * W, x[k], tau);
-    group_sync<G, WARPS>(tau);
+    group_sync<G, WARPS>(tau, th);
 #pragma unroll
     for (int k = 0; k < NP; ++k) xb_load<LOGN, E, S0B, HB>(xb + k * W, x[k], tau);
   } else {
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-      group_sync<G, WARPS>(tau);
+      group_sync<G, WARPS>(tau, th);
       xb_store<LOGN, E, S0A, HA>(xb, x[k], tau);
-      group_sync<G, WARPS>(tau);
+      group_sync<G, WARPS>(tau, th);
       xb_load<LOGN, E, S0B, HB>(xb, x[k], tau);
     }
   }
@@ -376,31 +459,32 @@ __device__ __forceinline__ void exchange(uint32_t (&x)[NP][E], uint32_t *xb, uin
 
 // Forward transform of NP polynomials held as x[k][e] = element
 // slot_index<LOGN,E,0,RAD>(tau, e) = tau + e*N/E of polynomial k.
-template <int LOGN, int E, int NP, int XBUF, bool P31 = false, int PASS = 0>
-__device__ __forceinline__ void ntt_forward(uint32_t (&x)[NP][E], const uint2 *tw, uint32_t *xb, uint32_t tau,
-                                            uint32_t p) {
+template <int LOGN, int E, int NP, int XBUF, bool P31 = false, int PASS = 0, class TW, class TH = CtaThreads>
+__device__ __forceinline__ void ntt_forward(uint32_t (&x)[NP][E], const TW &tw, uint32_t *xb, uint32_t tau,
+                                            uint32_t p, const TH &th = TH()) {
   using S = NttShape<LOGN, E>;
   constexpr int S0 = S::RAD * PASS;
   constexpr int H = S::template h<PASS>();
   fwd_pass<LOGN, E, NP, S0, H, P31>(x, tw, tau, p, 2 * p, 8 * p);
   if constexpr (PASS + 1 < S::NPASS) {
-    exchange<LOGN, E, NP, XBUF, S0, H, S0 + S::RAD, S::template h<PASS + 1>()>(x, xb, tau);
-    ntt_forward<LOGN, E, NP, XBUF, P31, PASS + 1>(x, tw, xb, tau, p);
+    exchange<LOGN, E, NP, XBUF, S0, H, S0 + S::RAD, S::template h<PASS + 1>()>(x, xb, tau, th);
+    ntt_forward<LOGN, E, NP, XBUF, P31, PASS + 1>(x, tw, xb, tau, p, th);
   }
 }
 
 // Inverse transform (without the N^{-1} factor).  Input: x[k][e] holds
 // bit-reversed position E*tau + e; output: natural position tau + e*N/E.
-template <int LOGN, int E, int NP, int XBUF, bool P31 = false, int PASS = NttShape<LOGN, E>::NPASS - 1>
-__device__ __forceinline__ void ntt_inverse(uint32_t (&x)[NP][E], const uint2 *tw, uint32_t *xb, uint32_t tau,
-                                            uint32_t p) {
+template <int LOGN, int E, int NP, int XBUF, bool P31 = false, int PASS = NttShape<LOGN, E>::NPASS - 1,
+          class TW, class TH = CtaThreads>
+__device__ __forceinline__ void ntt_inverse(uint32_t (&x)[NP][E], const TW &tw, uint32_t *xb, uint32_t tau,
+                                            uint32_t p, const TH &th = TH()) {
   using S = NttShape<LOGN, E>;
   constexpr int S0 = S::RAD * PASS;
   constexpr int H = S::template h<PASS>();
   inv_pass<LOGN, E, NP, S0, H, P31>(x, tw, tau, p, 8 * p);
   if constexpr (PASS > 0) {
-    exchange<LOGN, E, NP, XBUF, S0, H, S0 - S::RAD, S::RAD>(x, xb, tau);
-    ntt_inverse<LOGN, E, NP, XBUF, P31, PASS - 1>(x, tw, xb, tau, p);
+    exchange<LOGN, E, NP, XBUF, S0, H, S0 - S::RAD, S::RAD>(x, xb, tau, th);
+    ntt_inverse<LOGN, E, NP, XBUF, P31, PASS - 1>(x, tw, xb, tau, p, th);
   }
 }
 

@@ -63,6 +63,14 @@ bool fits_three_primes(const rosetta_params &p) {
   return bound * 20 <= M3 * 9;
 }
 
+// Does that bound stay within 2^kQfBits, where the float quotient's estimate is
+// good enough?
+bool fits_float_quotient(const rosetta_params &p) {
+  using u128 = unsigned __int128;
+  const u128 f = static_cast<u128>(p.glwe_dim + 1) * p.pbs_level * p.poly_size;
+  return (f << (p.pbs_base_log - 1 + 63)) <= (static_cast<u128>(1) << kQfBits);
+}
+
 int check_params(const rosetta_params &p) {
   const uint32_t logN = log2_exact(p.poly_size);
   if (logN < 8 || logN > 13) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
@@ -263,7 +271,47 @@ TraceArgs trace_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, u
   return a;
 }
 
+// Ciphertexts [first, first + count) of a launch.
+BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) {
+  a.lwe_in += first * lwe_words(c);
+  if (a.lwe_big_out) a.lwe_big_out += first * big_words(c);
+  if (a.lut_index) a.lut_index += first;
+  if (a.glwe_in) a.glwe_in += first * 2 * (size_t)c->prm.poly_size;
+  if (a.glwe_out) a.glwe_out += first * 2 * (size_t)c->prm.poly_size;
+  a.batch = count;
+  return a;
+}
+
 }  // namespace
+
+// Blind rotation of a batch: the cluster kernels, or at the standard ring, where
+// the context holds the float quotient's key, one worker per ciphertext for
+// whatever part of the batch fills the GPU.  A launch of w workers per SM takes
+// the same time for any number of ciphertexts up to w S (S SMs; measured at
+// n = 742: 9.7, 14.5, 20.6 ms for w = 1, 2, 3), the cluster kernel about in
+// proportion to its number (95: 7.8, 114: 9.7, 152: 10.9, 190: 14.4, 228: 15.8,
+// 304: 19.9 ms; at 456 28.8).  So whole waves of 3 S go to three workers, and
+// the rest r to as many workers as it needs, except where the cluster kernel
+// is still ahead: r <= 3/4 S and S < r <= 5/4 S.
+cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t s) {
+  if (!c->br_qf) return launch_blind_rotate(a, c->logN, c->dig16, s);
+  const uint32_t S = c->sms, wave = 3 * S;
+  uint32_t full = a.batch / wave * wave, rest = a.batch - full;
+  if (rest > 2 * S) {
+    full = a.batch;
+    rest = 0;
+  }
+  const auto solo = [&](uint32_t first, uint32_t count, uint32_t workers) {
+    BrArgs q = br_slice(c, a, first, count);
+    br_solo_key_args(c, &q);
+    return launch_blind_rotate_solo(q, c->tw_qf_host.data(), workers, s);
+  };
+  cudaError_t e = full ? solo(0, full, 3) : cudaSuccess;
+  if (e != cudaSuccess || rest == 0) return e;
+  if (rest <= S - S / 4 || (rest > S && rest <= S + S / 4))
+    return launch_blind_rotate(br_slice(c, a, full, rest), c->logN, c->dig16, s);
+  return solo(full, rest, rest <= S ? 1 : 2);
+}
 
 extern "C" {
 
@@ -314,7 +362,9 @@ int rosetta_params_init(rosetta_ctx **out, const rosetta_params *p, int cuda_dev
   // it, the kernel exists for the ring size and level, and as many of its
   // CTAs fit an SM's shared memory as of the four-prime kernel's; over the
   // four 28-bit primes otherwise.
-  int smem_sm = 0, smem_rsv = 0;
+  int smem_sm = 0, smem_rsv = 0, sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cuda_device);
+  c->sms = sms > 0 ? sms : 1;
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, cuda_device);
   cudaDeviceGetAttribute(&smem_rsv, cudaDevAttrReservedSharedMemoryPerBlock, cuda_device);
   const size_t smem3 = br3_smem_bytes(logN, p->pbs_level, p->lwe_dim);
@@ -326,12 +376,33 @@ int rosetta_params_init(rosetta_ctx **out, const rosetta_params *p, int cuda_dev
     tw31.resize((size_t)kPrimes31 << logN);
     if (build_tables(logN, kPrimes31, tw31.data(), &c->cc31)) c->br_primes = kPrimes31;
   }
+  // Three of the 28-bit primes and the float quotient for the launches that
+  // fill the GPU, where the bound allows it and three workers fit an SM.
+  std::vector<uint2> &tw_qf = c->tw_qf_host;
+  std::vector<double2> tw_f64;
+  if (fits_float_quotient(*p) && br_solo_supported(logN, p->pbs_level, p->pbs_base_log) &&
+      br_solo_smem_bytes(p->lwe_dim, 3) <= (size_t)max_smem) {
+    tw_f64.resize((size_t)1 << (logN - 1));
+    if (build_tables(logN, kPrimes, nullptr, &c->cc_qf, kPrimesQf)) {
+      tw_qf = tw;  // the first three primes' twiddles; the fourth's place takes the pass table
+      build_cfft_tables(logN, reinterpret_cast<float4 *>(tw_qf.data() + ((size_t)kPrimesQf << logN)), tw_f64.data());
+      c->br_qf = true;
+    }
+  }
   cudaError_t e = cudaMalloc(&c->d_tw, tw.size() * sizeof(uint2));
   if (e == cudaSuccess) e = cudaMemcpy(c->d_tw, tw.data(), tw.size() * sizeof(uint2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && c->br_primes == kPrimes31) {
     e = cudaMalloc(&c->d_tw31, tw31.size() * sizeof(uint2));
     if (e == cudaSuccess)
       e = cudaMemcpy(c->d_tw31, tw31.data(), tw31.size() * sizeof(uint2), cudaMemcpyHostToDevice);
+  }
+  if (e == cudaSuccess && c->br_qf) {
+    e = cudaMalloc(&c->d_tw_qf, tw_qf.size() * sizeof(uint2));
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_tw_f64, tw_f64.size() * sizeof(double2));
+    if (e == cudaSuccess)
+      e = cudaMemcpy(c->d_tw_qf, tw_qf.data(), tw_qf.size() * sizeof(uint2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(c->d_tw_f64, tw_f64.data(), tw_f64.size() * sizeof(double2), cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess) e = cudaMalloc(&c->d_lut, sizeof(uint64_t) << p->msg_bits);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_err, sizeof(uint32_t));
@@ -376,12 +447,16 @@ int rosetta_upload_bsk(rosetta_ctx *c, const uint64_t *bsk, size_t n_words, int 
   // one 32-bit residue per prime of the blind rotation's set for every raw word
   const bool three = c->br_primes == kPrimes31;
   if (!c->d_bsk) e = cudaMalloc(&c->d_bsk, want * c->br_primes * sizeof(uint32_t));
+  if (e == cudaSuccess && c->br_qf && !c->d_bsk_qf) e = cudaMalloc(&c->d_bsk_qf, want * kPrimes * sizeof(uint32_t));
   if (e != cudaSuccess) {
     if (tmp) cudaFreeAsync(tmp, s);
     return cuda_fail(e);
   }
   e = launch_bsk_transform(src, c->d_bsk, three ? c->d_tw31 : c->d_tw, three ? c->cc31 : c->cc, c->logN, p.lwe_dim,
                            p.pbs_level, c->br_primes, s);
+  if (e == cudaSuccess && c->br_qf)
+    e = launch_bsk_transform_qf(src, c->d_bsk_qf, c->d_tw_qf, c->d_tw_f64, c->cc_qf, c->logN, p.lwe_dim, p.pbs_level,
+                                s);
   if (tmp) cudaFreeAsync(tmp, s);
   if (e != cudaSuccess) return cuda_fail(e);
   if (!src_is_device) {
@@ -436,7 +511,7 @@ int rosetta_blind_rotate_extract_batch(rosetta_ctx *c, const uint64_t *lwe_in, u
   Staged st;
   int r = stage_io(c, lwe_in, lwe_words(c), batch, lut, lwe_big_out, big_words(c), s, &st);
   if (r != ROSETTA_OK) return r;
-  cudaError_t e = launch_blind_rotate(br_args(c, st.in, batch, st.lut, st.out), c->logN, c->dig16, s);
+  cudaError_t e = run_blind_rotate(c, br_args(c, st.in, batch, st.lut, st.out), s);
   if (e != cudaSuccess) return cuda_fail(e);
   return finish_io(c, lwe_big_out, big_words(c), batch, st, s);
 }
@@ -470,7 +545,7 @@ int rosetta_pbs_batch(rosetta_ctx *c, const uint64_t *lwe_in, uint32_t batch, co
   if (r != ROSETTA_OK) return r;
   r = ensure_big(c, batch, s);
   if (r != ROSETTA_OK) return r;
-  cudaError_t e = launch_blind_rotate(br_args(c, st.in, batch, st.lut, c->d_big), c->logN, c->dig16, s);
+  cudaError_t e = run_blind_rotate(c, br_args(c, st.in, batch, st.lut, c->d_big), s);
   if (e != cudaSuccess) return cuda_fail(e);
   e = run_keyswitch(c, c->d_big, batch, st.out, s);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -497,7 +572,7 @@ int rosetta_pbs_batch_multi_lut(rosetta_ctx *c, const uint64_t *lwe_in, uint32_t
   BrArgs a = br_args(c, st.in, batch, luts, c->d_big);
   a.lut_index = lut_index;
   a.num_luts = num_luts;
-  cudaError_t e = launch_blind_rotate(a, c->logN, c->dig16, s);
+  cudaError_t e = run_blind_rotate(c, a, s);
   if (e != cudaSuccess) return cuda_fail(e);
   e = run_keyswitch(c, c->d_big, batch, st.out, s);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -521,7 +596,7 @@ int rosetta_blind_rotate_glwe_batch(rosetta_ctx *c, const uint64_t *lwe_in, uint
   BrArgs a = br_args(c, lwe_in, batch, nullptr, nullptr);
   a.glwe_in = glwe_in;
   a.glwe_out = glwe_out;
-  cudaError_t e = launch_blind_rotate(a, c->logN, c->dig16, as_stream(stream));
+  cudaError_t e = run_blind_rotate(c, a, as_stream(stream));
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
 }
 
@@ -704,7 +779,7 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
   if (e == cudaSuccess) {
     BrArgs a = br_args(c, lwe_seg, batch, nullptr, c->d_big);
     a.glwe_in = T;
-    e = launch_blind_rotate(a, c->logN, c->dig16, s);
+    e = run_blind_rotate(c, a, s);
   }
   if (e == cudaSuccess) e = run_keyswitch(c, c->d_big, batch, I, s);
   // Step 3, phase 1: r_s = a_s(X) [[x]] + b_s(X), rotated by [[I]], traced, and
@@ -716,7 +791,7 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
       BrArgs a = br_args(c, I, batch, nullptr, nullptr);
       a.glwe_in = T;
       a.glwe_out = U;
-      e = launch_blind_rotate(a, c->logN, c->dig16, s);
+      e = run_blind_rotate(c, a, s);
     }
     if (e == cudaSuccess) e = launch_trace(trace_args(c, U, batch, T), c->logN, s);
     if (e == cudaSuccess) e = launch_monomial_acc(R, T, 2 * batch, c->logN, sg * seg_box, sg == 0, s);
@@ -727,7 +802,7 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
     BrArgs a = br_args(c, lwe_seg, batch, nullptr, nullptr);
     a.glwe_in = T;
     a.glwe_out = U;
-    e = launch_blind_rotate(a, c->logN, c->dig16, s);
+    e = run_blind_rotate(c, a, s);
   }
   if (e == cudaSuccess) e = launch_trace(trace_args(c, U, batch, glwe_out), c->logN, s);
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
@@ -786,7 +861,7 @@ int rosetta_selftest_bounds(rosetta_ctx *c, void *stream) {
   BrArgs a = br_args(c, c->d_in, 1, c->d_lut, c->d_big);
   const size_t step = c->bsk_words / c->prm.lwe_dim;
   a.bsk_words = c->bsk_words - step;
-  e = launch_blind_rotate(a, c->logN, c->dig16, s);
+  e = run_blind_rotate(c, a, s);
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
 #endif
 }
@@ -797,6 +872,9 @@ void rosetta_destroy(rosetta_ctx *c) {
   cudaDeviceSynchronize();
   cudaFree(c->d_tw);
   cudaFree(c->d_tw31);
+  cudaFree(c->d_tw_qf);
+  cudaFree(c->d_bsk_qf);
+  cudaFree(c->d_tw_f64);
   cudaFree(c->d_bsk);
   cudaFree(c->d_ksk);
   cudaFree(c->d_corr);

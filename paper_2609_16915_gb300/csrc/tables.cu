@@ -1,8 +1,10 @@
 // Host-side precomputation: twiddle tables and CRT constants for a set of NTT
 // primes (the four 28-bit primes, or the three 31-bit ones).  Runs once per
 // context and set.
+#include <cmath>
 #include <vector>
 
+#include "cfft.cuh"
 #include "internal.h"
 
 namespace rosetta {
@@ -61,9 +63,10 @@ uint32_t shoup(uint32_t w, uint32_t p) { return static_cast<uint32_t>((static_ca
 
 }  // namespace
 
-bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host, CrtConsts *cc) {
+bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host, CrtConsts *cc, uint32_t use) {
   const uint32_t N = 1u << logN;
-  if (primes != kPrimes && primes != kPrimes31) return false;
+  if ((primes != kPrimes && primes != kPrimes31) || use > primes) return false;
+  if (use == 0) use = primes;
   const uint32_t *list = primes == kPrimes ? kPrimeList : kPrime31List;
   // 28-bit set in (2^28 - 2^18, 2^28): lazy residues up to 16p fit 32 bits and
   // the CRT quotient may use 2^28 in place of p; 31-bit set in
@@ -71,18 +74,23 @@ bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host, CrtConsts *cc)
   const uint32_t top = primes == kPrimes ? 28 : 31, gap = primes == kPrimes ? 18 : 19;
   *cc = CrtConsts{};
   u128 M = 1;
-  for (uint32_t q = 0; q < primes; ++q) M *= list[q];
+  for (uint32_t q = 0; q < use; ++q) M *= list[q];
   cc->M_mod64 = static_cast<uint64_t>(M);
-  for (uint32_t q = 0; q < primes; ++q) {
+  cc->qf_base = cc->M_mod64 << (31 - kQfShift);
+  for (uint32_t q = 0; q < use; ++q) {
     const uint32_t p = list[q];
     if (!is_prime(p) || (p - 1) % (2 * N) != 0 || p >= (1u << top) || p <= (1u << top) - (1u << gap)) return false;
     const uint32_t g = generator(p);
     if (!g) return false;
     const uint32_t psi = powmod(g, (p - 1) / (2 * N), p);  // primitive 2N-th root of unity
     if (powmod(psi, N, p) != p - 1) return false;
-    for (uint32_t m = 0; m < N; ++m) {
-      const uint32_t w = powmod(psi, bitrev(m, logN), p);
-      tw_host[(size_t)q * N + m] = make_uint2(w, shoup(w, p));
+    if (tw_host) {
+      uint64_t w = 1;  // psi^i, i = bitrev(m)
+      for (uint32_t i = 0; i < N; ++i) {
+        tw_host[(size_t)q * N + bitrev(i, logN)] =
+            make_uint2(static_cast<uint32_t>(w), shoup(static_cast<uint32_t>(w), p));
+        w = w * psi % p;
+      }
     }
     PrimeConsts &pc = cc->pr[q];
     pc.p = p;
@@ -101,6 +109,28 @@ bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host, CrtConsts *cc)
     pc.Mp_mod64 = static_cast<uint64_t>(Mq);
   }
   return true;
+}
+
+void build_cfft_tables(uint32_t logN, float4 *pass_tw, double2 *tw) {
+  const uint32_t logC = logN - 1, C = 1u << logC;
+  // group g of stage s splits X^len - w^2; exponents of w to the primitive
+  // 2N-th root exp(i pi / N): the root node X^C - i has C/2, a node with
+  // exponent e has children e/2 and e/2 + C (i times the first)
+  std::vector<uint32_t> e(C);
+  e[1] = C / 2;
+  for (uint32_t m = 1; 2 * m < C; ++m) {
+    e[2 * m] = e[m] / 2;
+    e[2 * m + 1] = e[m] / 2 + C;
+  }
+  const double step = std::acos(-1.0) / (1u << logN);
+  tw[0] = make_double2(1.0, 0.0);
+  for (uint32_t m = 1; m < C; ++m) tw[m] = make_double2(std::cos(step * e[m]), std::sin(step * e[m]));
+  for (uint32_t pass = 0; 2 * pass < logC; ++pass)
+    for (uint32_t g = 0; g < (1u << (2 * pass)); ++g) {
+      const double2 w1 = tw[(1u << (2 * pass)) + g], w2 = tw[(2u << (2 * pass)) + 2 * g];
+      pass_tw[cfft_tw_offset(pass) + g] = make_float4(static_cast<float>(w1.x), static_cast<float>(w1.y),
+                                                      static_cast<float>(w2.x), static_cast<float>(w2.y));
+    }
 }
 
 }  // namespace rosetta

@@ -97,8 +97,8 @@ typedef struct {
  * not fit the four NTT primes: log2((k+1) l N 2^(beta-1) 2^63) + 1 must not
  * exceed 111 (their product is about 2^111.99); and when one blind-rotation
  * CTA (a quarter of the ring) does not fit the device's shared memory per
- * block: 12N + max(8N, 4.5N per exchange buffer (two for N <= 1024, else
- * one)) + l N x {1 for beta <= 16 | 2} + 2(n+1) bytes, which on a 227 KB
+ * block: 12N + max(8N, 4.5N per exchange buffer (two for N <= 1024, and at
+ * N = 2048 with up to three levels, else one)) + l N x {1 for beta <= 16 | 2} + 2(n+1) bytes, which on a 227 KB
  * device admits at N = 8192, for example, l = 3 with beta <= 16 up to
  * n = 22015, l = 4 or l = 2 with beta > 16 up to n = 17919, and l = 3 with
  * beta > 16 up to n = 9727.  Errors: INVALID_ARG (NULL), UNSUPPORTED_PARAMS,

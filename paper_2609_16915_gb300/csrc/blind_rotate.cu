@@ -51,8 +51,11 @@ __host__ __device__ constexpr int br_xbuf(int logN) { return logN <= 10 ? 2 : 1;
 
 // Exchange-buffer words: the transforms' XBUF x (N + N/8), and at least 2N
 // (16 T) for the outgoing residues, four groups of four words per thread.
-__host__ __device__ constexpr int br_xb_words(int logN) {
-  return br_xbuf(logN) * ((1 << logN) + (1 << logN) / 8) > 2 * (1 << logN)
+// With `pairs` (the transforms exchange both polynomials of a pair as 8-byte
+// elements) 2 (N + N/8).
+__host__ __device__ constexpr int br_xb_words(int logN, bool pairs) {
+  return pairs ? 2 * ((1 << logN) + (1 << logN) / 8)
+         : br_xbuf(logN) * ((1 << logN) + (1 << logN) / 8) > 2 * (1 << logN)
              ? br_xbuf(logN) * ((1 << logN) + (1 << logN) / 8)
              : 2 * (1 << logN);
 }
@@ -62,6 +65,12 @@ __host__ __device__ constexpr int br_xb_words(int logN) {
 // (N = 2048: 309 vs 276 ms, 4096: 822 vs 782 ms, 8192: 14.0 vs 12.8 s for the
 // full batches), so 8 is used throughout.
 __host__ __device__ constexpr int br_e(int) { return 8; }
+
+// The compiled-level kernels of the standard ring exchange pairs and read the
+// first pass's twiddles from the constant bank (with the closed-form digits:
+// 5.51 -> 5.23 ms at 38 ciphertexts, 7.77 -> 7.38 at 77, 14.36 -> 13.56 at 190,
+// n = 742; one ciphertext, bound by latency, stays at 3.89).
+__host__ __device__ constexpr bool br_pairs(int logN, int level) { return logN == 11 && level >= 1 && level <= 3; }
 
 template <int LOGN>
 struct BrShape {
@@ -77,16 +86,32 @@ struct BrShape {
   static constexpr int MIN_CTAS = (LOGN <= 11) ? 4 : (LOGN == 12 ? 2 : 1);
 };
 
+template <int LOGN, bool SPLIT>
+__device__ __forceinline__ uint32_t tw_slot(uint32_t m) {
+  if constexpr (SPLIT) return split_tw_slot<LOGN>(m);
+  return m;
+}
+template <int LOGN, bool SPLIT>
+__device__ __forceinline__ auto make_tw(const uint2 *sm, const uint2 *cst) {
+  if constexpr (SPLIT)
+    return SplitTw<LOGN, 3>{sm, cst};
+  else
+    return sm;
+}
+
 // LEV > 0 fixes the gadget level count at compile time (the common sets:
 // straight-line digit and key loops); LEV = 0 reads it from the arguments.
 template <int LOGN, bool DIG16, int LEV>
-__global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) blind_rotate_kernel(const BrArgs a) {
+__global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) blind_rotate_kernel(const __grid_constant__ BrArgs a) {
   using B = BrShape<LOGN>;
   using S = NttShape<LOGN, B::E>;
   using DigT = typename std::conditional<DIG16, int16_t, int32_t>::type;
   constexpr uint32_t N = B::N, T = B::T, Q = B::Q;
   constexpr int E = B::E, ITEMS = B::ITEMS, QE = B::QE;
   constexpr uint32_t TWO_N = 2 * N;
+  constexpr bool PAIRS = br_pairs(LOGN, LEV);
+  constexpr int XBUF = PAIRS ? 2 : B::XBUF;
+  using TH = typename std::conditional<PAIRS, CtaPairs, CtaThreads>::type;
 
   cg::cluster_group cluster = cg::this_cluster();
   const uint32_t rank = cluster.block_rank();
@@ -95,13 +120,14 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
   if (!dbg_ok(ct < a.batch, a.err_flag)) return;  // the whole cluster shares ct
 
   extern __shared__ __align__(16) unsigned char smem[];
-  uint2 *tw = reinterpret_cast<uint2 *>(smem);                   // [N]
-  uint64_t *acc = reinterpret_cast<uint64_t *>(tw + N);          // [2][Q]
+  uint2 *tw_s = reinterpret_cast<uint2 *>(smem);                 // [N]
+  uint64_t *acc = reinterpret_cast<uint64_t *>(tw_s + N);          // [2][Q]
   // [XBUF][XB_WORDS] for the transforms; after the inverse transforms the
   // outgoing residues [owner][T][2 comp][QE halves]
   uint32_t *xb = reinterpret_cast<uint32_t *>(acc + 2 * Q);
-  static_assert(br_xb_words(LOGN) >= B::XBUF * S::XB_WORDS, "exchange buffer");
-  DigT *dig = reinterpret_cast<DigT *>(xb + br_xb_words(LOGN));  // [l row pairs][T][2][QE]
+  constexpr int XB_WORDS = br_xb_words(LOGN, PAIRS);
+  static_assert(XB_WORDS >= XBUF * S::XB_WORDS, "exchange buffer");
+  DigT *dig = reinterpret_cast<DigT *>(xb + XB_WORDS);  // [l row pairs][T][2][QE]
   const uint32_t level = LEV > 0 ? static_cast<uint32_t>(LEV) : a.level;
   uint16_t *atil = reinterpret_cast<uint16_t *>(dig + 2 * level * Q);  // [n+1]
 
@@ -109,7 +135,8 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
   const uint32_t p_inv = a.cc.pr[rank].p_inv;
 
   // ---- set-up: twiddles, modulus switch, accumulator ----
-  for (uint32_t m = tau; m < N; m += T) tw[m] = a.tw[rank * N + m];
+  for (uint32_t m = tau; m < N; m += T) tw_s[tw_slot<LOGN, PAIRS>(m)] = a.tw[rank * N + m];
+  const auto tw = make_tw<LOGN, PAIRS>(tw_s, a.tw_lo[rank]);
   const uint64_t *lwe = a.lwe_in + static_cast<size_t>(ct) * (a.n + 1);
   constexpr uint32_t SH = 63 - LOGN;  // 64 - log2(2N)
   for (uint32_t i = tau; i <= a.n; i += T)
@@ -162,11 +189,8 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
   // in another CTA of the cluster
   const uint32_t acc_s = smem_addr(acc), dig_s = smem_addr(dig), xb_s = smem_addr(xb);
   const uint32_t L2 = 2 * level;
-  const uint32_t bits = a.base_log * level;
-  const uint64_t Bmask = (1ull << a.base_log) - 1;
-  const uint64_t Bhalf = 1ull << (a.base_log - 1);
-  const uint64_t round_add = bits >= 64 ? 0 : (1ull << (63 - bits));
-  const uint32_t round_sh = bits >= 64 ? 0 : 64 - bits;
+  const uint64_t dig_add = dig_offset(a.base_log, level);
+  const int32_t dig_half = 1 << (a.base_log - 1);
 
   // Packed exchange layouts.  Owner thread tau holds the items (c, jl) =
   // (m / QE, tau + (m % QE) T), m < ITEMS = 2 QE, and prime thread tau needs
@@ -216,17 +240,10 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
       const uint32_t item = tau + m * T;
       const uint32_t c = item / Q, jl = item % Q, j = rank * Q + jl;
       const bool neg = ((j + TWO_N - at) & (TWO_N - 1)) >= N;
-      const uint64_t diff = (neg ? 0ull - v[m] : v[m]) - acc[c * Q + jl];
-      uint64_t cv = bits >= 64 ? diff : (diff + round_add) >> round_sh;
+      const uint64_t w = (neg ? 0ull - v[m] : v[m]) - acc[c * Q + jl] + dig_add;
 #pragma unroll
-      for (int l = static_cast<int>(level) - 1; l >= 0; --l) {
-        const uint64_t d = cv & Bmask;
-        cv >>= a.base_log;
-        int32_t ds = static_cast<int32_t>(d);
-        if (d >= Bhalf) {
-          ds -= static_cast<int32_t>(Bmask + 1);
-          cv += 1;
-        }
+      for (int l = 0; l < static_cast<int>(level); ++l) {
+        const int32_t ds = static_cast<int32_t>(biased_digit(w, a.base_log, l)) - dig_half;
         const uint32_t r = c * level + l;  // row; h = m % QE
         if constexpr (LEV > 0)
           grp[r >> 1][(r & 1) * QE + (m % QE)] = ds;
@@ -291,7 +308,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
           for (int h = 0; h < QE; ++h)
             x[pp][o * QE + h] = static_cast<uint32_t>(d[pp * QE + h] + static_cast<int32_t>(p));  // in (0, 2p)
       }
-      ntt_forward<LOGN, E, 2, B::XBUF>(x, tw, xb, tau, p);
+      ntt_forward<LOGN, E, 2, XBUF>(x, tw, xb, tau, p, TH());
       // BSK_i words of this prime for rows r0, r0+1, E per thread and
       // component, contiguous across the CTA (16-byte loads)
       const uint4 *g = reinterpret_cast<const uint4 *>(gbase + static_cast<size_t>(r0) * 2 * N + E * tau);
@@ -321,7 +338,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
         }
       }
     }
-    ntt_inverse<LOGN, E, 2, B::XBUF>(oh, tw, xb, tau, p);
+    ntt_inverse<LOGN, E, 2, XBUF>(oh, tw, xb, tau, p, TH());
     __syncthreads();  // every exchange read done: the buffer takes the outgoing residues
     // CRT-scaled residues (< 8p; the keys carry the CRT factor), one packed
     // group (component, h) per owner
@@ -394,7 +411,8 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
 
 size_t br_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, bool dig16) {
   const size_t N = size_t(1) << logN, Q = N / 4;
-  size_t b = N * sizeof(uint2) + 2 * Q * sizeof(uint64_t) + br_xb_words(static_cast<int>(logN)) * sizeof(uint32_t) +
+  size_t b = N * sizeof(uint2) + 2 * Q * sizeof(uint64_t) +
+             br_xb_words(static_cast<int>(logN), br_pairs(static_cast<int>(logN), static_cast<int>(level))) * sizeof(uint32_t) +
              2 * level * Q * (dig16 ? 2 : 4) + (n + 1) * sizeof(uint16_t);
   return (b + 15) & ~size_t(15);
 }

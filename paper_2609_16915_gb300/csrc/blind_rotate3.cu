@@ -23,10 +23,20 @@
 //     own exchange buffer, from which the owners read them in phase 3.
 // Every cross-CTA read follows a write to the writer's own shared memory, so
 // the step's barriers order shared memory only (cluster_sync_shared).
+// Where the shared memory takes it without costing a resident CTA (PAIRS; every
+// n up to a few thousand), the two polynomials of a row pair cross the exchange
+// buffer as 8-byte pairs: half the shared-memory instructions and barriers, and
+// no bank conflicts at N = 8192's stride-2 pass.  The first pass's twiddles come
+// from the constant bank, and digits are cut in closed form (biased_digit).
+// Measured: n = 840, N = 4096, l = 2, batch 1216: 228.7 ms before, 222.5 with
+// pairs and constant twiddles, 214.5 with the digits; n = 900, N = 8192, l = 3,
+// batch 152: 117.4, 113.4, 111.9 ms.
 // Per ciphertext and step the cluster runs 3 (l + 1) x 2 transforms instead
 // of 4 (l + 1) x 2; a butterfly is seven instructions instead of five and,
 // measured alone, about 15 % slower.
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "check.cuh"
 #include "dsmem.cuh"
@@ -53,38 +63,39 @@ struct Br3Shape {
   // resident CTAs per SM the register allocation must allow (2 x 92-98 KB of
   // shared memory at N = 4096, 1 x 198 KB at 8192)
   static constexpr int MIN_CTAS = LOGN <= 12 ? 2 : 1;
-  // exchange buffer words: N + N/8 for the transforms, extended to 12 T so
-  // that it holds the outgoing residues afterwards
-  static constexpr int XB_WORDS = 12 * T;
+  // exchange buffer words: N + N/8 for the transforms (twice that when pairs
+  // of words travel), extended to 12 T so that it holds the outgoing residues
+  // afterwards
+  template <bool PAIRS>
+  __host__ __device__ static constexpr int xb_words() { return PAIRS ? 18 * T : 12 * T; }
 };
 
-__device__ __forceinline__ uint32_t pack16(int32_t lo, int32_t hi) {
-  return (static_cast<uint32_t>(lo) & 0xFFFFu) | (static_cast<uint32_t>(hi) << 16);
-}
-__device__ __forceinline__ int32_t lo16(uint32_t w) { return static_cast<int16_t>(w & 0xFFFFu); }
-__device__ __forceinline__ int32_t hi16(uint32_t w) { return static_cast<int16_t>(w >> 16); }
+__device__ __forceinline__ uint32_t pack16(uint32_t lo, uint32_t hi) { return lo | (hi << 16); }  // both < 2^16
+__device__ __forceinline__ uint32_t lo16(uint32_t w) { return w & 0xFFFFu; }
+__device__ __forceinline__ uint32_t hi16(uint32_t w) { return w >> 16; }
 
 }  // namespace
 
 // Shared memory, in this order (16-byte aligned pieces):
 //   tw    uint2  [N]           twiddles of prime `rank`
 //   acc   uint64 [2][3][T]     owned accumulator words (component, slot, thread)
-//   xb    uint32 [12 T]        transform exchange buffer (N + N/8 words); after the
+//   xb    uint32 [12 T]        transform exchange buffer (N + N/8 words; 18 T words for
+//                              2N + N/4 with PAIRS); after the
 //                              inverse transforms the outgoing residues: [2 other
 //                              owners][T][4] (slots 0, 1 of both components), then
 //                              [2][T][2] (slot 2, owners 0 and 1)
-//   dig8  uint32 [l][T][2]     16-bit digits of each row pair: slots 0, 1 of both rows
+//   dig8  uint32 [l][T][2]     16-bit digits (plus B/2) of each row pair: slots 0, 1 of both rows
 //   dig4  uint32 [l][T]        slot 2 of both rows (owners 0 and 1)
 //   atil  uint16 [n+1]         switched mask and body
-size_t br3_smem_bytes(uint32_t logN, uint32_t level, uint32_t n) {
+size_t br3_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, bool pairs) {
   const size_t N = size_t(1) << logN, T = N / 8;
-  size_t b = N * sizeof(uint2) + 6 * T * sizeof(uint64_t) + (12 * T + 3 * level * T) * sizeof(uint32_t) +
+  size_t b = N * sizeof(uint2) + 6 * T * sizeof(uint64_t) + ((pairs ? 18 : 12) * T + 3 * level * T) * sizeof(uint32_t) +
              (n + 1) * sizeof(uint16_t);
   return (b + 15) & ~size_t(15);
 }
 
-template <int LOGN, int LEV>
-__global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) blind_rotate3_kernel(const BrArgs a) {
+template <int LOGN, int LEV, bool PAIRS>
+__global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) blind_rotate3_kernel(const __grid_constant__ BrArgs a) {
   using B = Br3Shape<LOGN>;
   using S = NttShape<LOGN, 8>;
   constexpr uint32_t N = B::N, T = B::T, TWO_N = 2 * N;
@@ -98,11 +109,14 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
   if (!dbg_ok(ct < a.batch, a.err_flag)) return;  // the whole cluster shares ct
 
   extern __shared__ __align__(16) unsigned char smem[];
-  static_assert(B::XB_WORDS >= S::XB_WORDS, "exchange buffer");
-  uint2 *tw = reinterpret_cast<uint2 *>(smem);
-  uint64_t *acc = reinterpret_cast<uint64_t *>(tw + N);
+  constexpr int XB_WORDS = B::template xb_words<PAIRS>();
+  static_assert(XB_WORDS >= (PAIRS ? 2 : 1) * S::XB_WORDS, "exchange buffer");
+  using TH = typename std::conditional<PAIRS, CtaPairs, CtaThreads>::type;
+  constexpr int XBUF = PAIRS ? 2 : 1;
+  uint2 *tw_s = reinterpret_cast<uint2 *>(smem);
+  uint64_t *acc = reinterpret_cast<uint64_t *>(tw_s + N);
   uint32_t *xb = reinterpret_cast<uint32_t *>(acc + 6 * T);
-  uint32_t *dig8 = xb + B::XB_WORDS;
+  uint32_t *dig8 = xb + XB_WORDS;
   uint32_t *dig4 = dig8 + L * T * 2;
   uint16_t *atil = reinterpret_cast<uint16_t *>(dig4 + L * T);
 
@@ -112,7 +126,8 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
   const bool three = rank < 2;    // owners 0 and 1 hold a third slot
 
   // ---- set-up: twiddles, modulus switch, accumulator ----
-  for (uint32_t m = tau; m < N; m += T) tw[m] = a.tw[rank * N + m];
+  for (uint32_t m = tau; m < N; m += T) tw_s[split_tw_slot<LOGN>(m)] = a.tw[rank * N + m];
+  const SplitTw<LOGN, 3> tw{tw_s, a.tw_lo[rank]};
   const uint64_t *lwe = a.lwe_in + static_cast<size_t>(ct) * (a.n + 1);
   constexpr uint32_t SH = 63 - LOGN;  // 64 - log2(2N)
   for (uint32_t i = tau; i <= a.n; i += T)
@@ -162,11 +177,8 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
 
   const uint32_t acc_s = smem_addr(acc), dig8_s = smem_addr(dig8), dig4_s = smem_addr(dig4);
   const uint32_t xb_s = smem_addr(xb);
-  const uint32_t bits = a.base_log * L;
-  const uint64_t Bmask = (1ull << a.base_log) - 1;
-  const uint64_t Bhalf = 1ull << (a.base_log - 1);
-  const uint64_t round_add = bits >= 64 ? 0 : (1ull << (63 - bits));
-  const uint32_t round_sh = bits >= 64 ? 0 : 64 - bits;
+  const uint64_t dig_add = dig_offset(a.base_log, L);
+  const uint32_t dig_bias = p - (1u << (a.base_log - 1));  // stored digits lie in [0, B): d + p = stored + bias
 
   for (uint32_t i = 0; i < a.n; ++i) {
     const uint32_t at = atil[i];
@@ -187,7 +199,7 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
         if (hg == 1 && !three) break;
         constexpr int NS_MAX = 2;
         const int h0 = hg == 0 ? 0 : 2, ns = hg == 0 ? 2 : 1;
-        int32_t g[L][2][NS_MAX];  // [row pair][row parity][slot of the group]
+        uint32_t g[L][2][NS_MAX];  // [row pair][row parity][slot of the group]
         uint64_t v[2][NS_MAX];
 #pragma unroll
         for (int c = 0; c < 2; ++c)
@@ -207,19 +219,11 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
             const int h = h0 + k;
             const uint32_t j = tau + (s0 + h) * T;
             const bool neg = ((j + TWO_N - at) & (TWO_N - 1)) >= N;
-            const uint64_t diff = (neg ? 0ull - v[c][k] : v[c][k]) - acc[(c * 3 + h) * T + tau];
-            uint64_t cv = bits >= 64 ? diff : (diff + round_add) >> round_sh;
+            const uint64_t diff = (neg ? 0ull - v[c][k] : v[c][k]) - acc[(c * 3 + h) * T + tau] + dig_add;
 #pragma unroll
-            for (int l = static_cast<int>(L) - 1; l >= 0; --l) {
-              const uint64_t d = cv & Bmask;
-              cv >>= a.base_log;
-              int32_t ds = static_cast<int32_t>(d);
-              if (d >= Bhalf) {
-                ds -= static_cast<int32_t>(Bmask + 1);
-                cv += 1;
-              }
+            for (int l = 0; l < static_cast<int>(L); ++l) {
               const int r = c * static_cast<int>(L) + l;
-              g[r >> 1][r & 1][k] = ds;
+              g[r >> 1][r & 1][k] = biased_digit(diff, a.base_log, l);
             }
           }
 #pragma unroll
@@ -232,7 +236,7 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
         }
       }
     } else {
-      int32_t g[L][2][3];  // [row pair][row parity][slot]
+      uint32_t g[L][2][3];  // [row pair][row parity][slot]
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint64_t v[3];
@@ -249,19 +253,11 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
           if (h == 2 && !three) continue;
           const uint32_t j = tau + (s0 + h) * T;
           const bool neg = ((j + TWO_N - at) & (TWO_N - 1)) >= N;
-          const uint64_t diff = (neg ? 0ull - v[h] : v[h]) - acc[(c * 3 + h) * T + tau];
-          uint64_t cv = bits >= 64 ? diff : (diff + round_add) >> round_sh;
+          const uint64_t diff = (neg ? 0ull - v[h] : v[h]) - acc[(c * 3 + h) * T + tau] + dig_add;
 #pragma unroll
-          for (int l = static_cast<int>(L) - 1; l >= 0; --l) {
-            const uint64_t d = cv & Bmask;
-            cv >>= a.base_log;
-            int32_t ds = static_cast<int32_t>(d);
-            if (d >= Bhalf) {
-              ds -= static_cast<int32_t>(Bmask + 1);
-              cv += 1;
-            }
+          for (int l = 0; l < static_cast<int>(L); ++l) {
             const int r = c * static_cast<int>(L) + l;
-            g[r >> 1][r & 1][h] = ds;
+            g[r >> 1][r & 1][h] = biased_digit(diff, a.base_log, l);
           }
         }
 #pragma unroll
@@ -291,17 +287,17 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
       for (int o = 0; o < 3; ++o) {
         const uint32_t q = own_s0(o);
         const uint2 w = dsmem_ld_v2_u32(dsmem_map(dig8_s + (P * T + tau) * 8u, o));
-        x[0][q] = static_cast<uint32_t>(lo16(w.x)) + p;  // (0, 2p)
-        x[0][q + 1] = static_cast<uint32_t>(hi16(w.x)) + p;
-        x[1][q] = static_cast<uint32_t>(lo16(w.y)) + p;
-        x[1][q + 1] = static_cast<uint32_t>(hi16(w.y)) + p;
+        x[0][q] = lo16(w.x) + dig_bias;  // (0, 2p)
+        x[0][q + 1] = hi16(w.x) + dig_bias;
+        x[1][q] = lo16(w.y) + dig_bias;
+        x[1][q + 1] = hi16(w.y) + dig_bias;
         if (o < 2) {
           const uint32_t w4 = dsmem_ld_u32(dsmem_map(dig4_s + (P * T + tau) * 4u, o));
-          x[0][q + 2] = static_cast<uint32_t>(lo16(w4)) + p;
-          x[1][q + 2] = static_cast<uint32_t>(hi16(w4)) + p;
+          x[0][q + 2] = lo16(w4) + dig_bias;
+          x[1][q + 2] = hi16(w4) + dig_bias;
         }
       }
-      ntt_forward<LOGN, E, 2, 1, true>(x, tw, xb, tau, p);  // outputs in [0, 2p)
+      ntt_forward<LOGN, E, 2, XBUF, true>(x, tw, xb, tau, p, TH());  // outputs in [0, 2p)
       // below p, so that a row pair's two products sum below 2 p^2 < p 2^32
 #pragma unroll
       for (int pp = 0; pp < 2; ++pp)
@@ -328,7 +324,7 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
         }
       }
     }
-    ntt_inverse<LOGN, E, 2, 1, true>(oh, tw, xb, tau, p);  // outputs in [0, 2p)
+    ntt_inverse<LOGN, E, 2, XBUF, true>(oh, tw, xb, tau, p, TH());  // outputs in [0, 2p)
     // CRT-scaled residues (the keys carry the CRT factor): one packed group
     // per other owner, left in this CTA's exchange buffer (once every thread
     // has finished the transforms' last exchange) at the owner's index among
@@ -414,10 +410,10 @@ bool br3_supported(uint32_t logN, uint32_t level, bool dig16) {
   return dig16 && (logN == 12 || logN == 13) && level >= 1 && level <= 3;
 }
 
-template <int LOGN, int LEV>
+template <int LOGN, int LEV, bool PAIRS>
 static cudaError_t launch_br3_t(const BrArgs &a, cudaStream_t s) {
-  auto kern = blind_rotate3_kernel<LOGN, LEV>;
-  const size_t smem = br3_smem_bytes(LOGN, LEV, a.n);
+  auto kern = blind_rotate3_kernel<LOGN, LEV, PAIRS>;
+  const size_t smem = br3_smem_bytes(LOGN, LEV, a.n, PAIRS);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -439,20 +435,19 @@ static cudaError_t launch_br3_t(const BrArgs &a, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
+template <int LOGN, bool PAIRS>
+static cudaError_t launch_br3_lev(const BrArgs &a, cudaStream_t s) {
+  switch (a.level) {
+    case 1: return launch_br3_t<LOGN, 1, PAIRS>(a, s);
+    case 2: return launch_br3_t<LOGN, 2, PAIRS>(a, s);
+    default: return launch_br3_t<LOGN, 3, PAIRS>(a, s);
+  }
+}
+
 cudaError_t launch_blind_rotate3(const BrArgs &a, uint32_t logN, cudaStream_t s) {
   if (a.primes != kPrimes31 || !br3_supported(logN, a.level, true)) return cudaErrorInvalidValue;
-  if (logN == 12) {
-    switch (a.level) {
-      case 1: return launch_br3_t<12, 1>(a, s);
-      case 2: return launch_br3_t<12, 2>(a, s);
-      default: return launch_br3_t<12, 3>(a, s);
-    }
-  }
-  switch (a.level) {
-    case 1: return launch_br3_t<13, 1>(a, s);
-    case 2: return launch_br3_t<13, 2>(a, s);
-    default: return launch_br3_t<13, 3>(a, s);
-  }
+  if (logN == 12) return a.pairs ? launch_br3_lev<12, true>(a, s) : launch_br3_lev<12, false>(a, s);
+  return a.pairs ? launch_br3_lev<13, true>(a, s) : launch_br3_lev<13, false>(a, s);
 }
 
 }  // namespace rosetta

@@ -42,14 +42,6 @@
 
 namespace rosetta {
 
-// Twiddles of one prime.  The first six stages' (64 entries, the same for a
-// whole warp) come from the constant bank, the others from shared memory; the
-// last stage's, four consecutive ones per thread, are stored as two runs of
-// pairs so that neighbouring threads' 16-byte loads touch neighbouring words.
-struct SoloTw {
-  const uint2 *sm, *cst;
-};
-
 namespace {
 
 constexpr int kLogN = 11;
@@ -58,15 +50,6 @@ constexpr uint32_t kWorkers = 3;                    // per CTA (and SM)
 constexpr uint32_t kTwF = 352;                      // float4 entries of the pass table (341, padded)
 constexpr uint32_t kXbWords = 2 * NttShape<kLogN, 8>::XB_WORDS;  // two integer polynomials; four float ones
 static_assert(kXbWords >= 4 * (kN / 2), "exchange buffer");
-
-constexpr int kConstStages = 6;
-struct SoloConstTw {
-  uint2 w[kPrimesQf][1 << kConstStages];
-};
-
-__device__ __forceinline__ uint32_t last_stage_slot(uint32_t idx) {  // idx in [N/2, N)
-  return kN / 2 + ((idx >> 1) & 1u) * (kN / 4) + (((idx - kN / 2) >> 2) << 1) + (idx & 1u);
-}
 
 __host__ __device__ constexpr size_t solo_worker_bytes(uint32_t n) {
   return 2 * kN * sizeof(uint64_t) + kXbWords * sizeof(uint32_t) + (((n + 1) * sizeof(uint16_t) + 15) & ~size_t(15));
@@ -88,34 +71,10 @@ __device__ __forceinline__ void add_residues(ulonglong2 *acc, const uint32_t (&y
   }
 }
 
-template <int S>
-__device__ __forceinline__ uint2 tw_at(const SoloTw &tw, uint32_t idx) {
-  if constexpr (S < kConstStages)
-    return tw.cst[idx];
-  else
-    return tw.sm[idx];
-}
-
-template <int S, int CNT>
-__device__ __forceinline__ void load_twiddles(const SoloTw &tw, uint32_t start, uint2 (&w)[CNT]) {
-  if constexpr (S == kLogN - 1) {
-    static_assert(CNT == 4, "four per thread in the last stage");
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const uint4 v = *reinterpret_cast<const uint4 *>(tw.sm + kN / 2 + k * (kN / 4) + (start - kN / 2) / 2);
-      w[2 * k] = make_uint2(v.x, v.y);
-      w[2 * k + 1] = make_uint2(v.z, v.w);
-    }
-  } else {
-    load_twiddles<S>(tw.sm, start, w);
-  }
-}
-
 // Shared memory: twiddles of the three primes uint2 [3][N], the float pass
 // table float4 [352], then per worker acc uint64 [N][2], the exchange buffer,
 // the switched mask and body uint16 [n+1].
-__global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(const __grid_constant__ BrArgs a,
-                                                                               const __grid_constant__ SoloConstTw ctw) {
+__global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(const __grid_constant__ BrArgs a) {
   constexpr uint32_t N = kN, T = kT, TWO_N = 2 * N;
   constexpr int E = 8;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -130,7 +89,7 @@ __global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(cons
 
   for (uint32_t m = threadIdx.x; m < kPrimesQf * N; m += blockDim.x) {
     const uint32_t q = m / N, idx = m % N;
-    tw_all[idx < N / 2 ? m : q * N + last_stage_slot(idx)] = a.tw[m];
+    tw_all[q * N + split_tw_slot<kLogN>(idx)] = a.tw[m];
   }
   const float4 *twf_src = reinterpret_cast<const float4 *>(a.tw + kPrimesQf * N);
   for (uint32_t m = threadIdx.x; m < kTwF; m += blockDim.x) twf[m] = twf_src[m];
@@ -217,7 +176,7 @@ __global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(cons
         q = q == kPrimesQf - 1 ? 0 : q + 1;
       }
       const uint32_t p = a.cc.pr[q].p, p_inv = a.cc.pr[q].p_inv;
-      const SoloTw tw{tw_all + q * N, ctw.w[q]};
+      const SplitTw<kLogN, 6> tw{tw_all + q * N, a.tw_lo[q]};
       uint32_t x[2][E];
 #pragma unroll
       for (int pp = 0; pp < 2; ++pp)
@@ -329,16 +288,13 @@ bool br_solo_supported(uint32_t logN, uint32_t level, uint32_t base_log) {
 
 size_t br_solo_smem_bytes(uint32_t n, uint32_t workers) { return solo_table_bytes() + workers * solo_worker_bytes(n); }
 
-cudaError_t launch_blind_rotate_solo(const BrArgs &a, const uint2 *tw_host, uint32_t workers, cudaStream_t s) {
+cudaError_t launch_blind_rotate_solo(const BrArgs &a, uint32_t workers, cudaStream_t s) {
   if (workers < 1 || workers > kWorkers) return cudaErrorInvalidValue;
   const size_t smem = br_solo_smem_bytes(a.n, workers);
   cudaError_t e = cudaFuncSetAttribute(blind_rotate_solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  SoloConstTw ctw;
-  for (int q = 0; q < kPrimesQf; ++q)
-    for (int m = 0; m < (1 << kConstStages); ++m) ctw.w[q][m] = tw_host[q * kN + m];
-  blind_rotate_solo_kernel<<<(a.batch + workers - 1) / workers, workers * kT, smem, s>>>(a, ctw);
+  blind_rotate_solo_kernel<<<(a.batch + workers - 1) / workers, workers * kT, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -4,8 +4,7 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
-
-#include <vector>
+#include <string.h>
 
 #include "rosetta.h"
 #include "internal.h"
@@ -21,6 +20,9 @@ struct rosetta_ctx {
   // the blind rotation's prime set: kPrimes (d_tw, cc) or, where the
   // external-product bound allows, the three 31-bit primes (d_tw31, cc31)
   uint32_t br_primes = rosetta::kPrimes;
+  bool br3_pairs = false;         // three primes: paired exchange buffer (fits as densely)
+  uint2 tw_lo[rosetta::kPrimes][rosetta::kTwLo] = {};     // first twiddles of the 28-bit set
+  uint2 tw_lo31[rosetta::kPrimes31][rosetta::kTwLo] = {};  // and of the 31-bit set
   uint2 *d_tw31 = nullptr;        // [kPrimes31][N], or null
   rosetta::CrtConsts cc31{};
   // the worker-per-ciphertext kernel of the standard ring (three 28-bit primes
@@ -28,7 +30,6 @@ struct rosetta_ctx {
   // primes' twiddles and the pass table [4][N], the key transform's table
   bool br_qf = false;
   uint2 *d_tw_qf = nullptr;
-  std::vector<uint2> tw_qf_host;
   double2 *d_tw_f64 = nullptr;    // [N/2]
   rosetta::CrtConsts cc_qf{};
   uint32_t *d_bsk_qf = nullptr;   // [n][4][2][2][N]
@@ -75,7 +76,9 @@ inline void br_key_args(const rosetta_ctx *c, rosetta::BrArgs *a) {
   a->bsk = c->d_bsk;
   a->bsk_words = c->bsk_words;
   a->primes = c->br_primes;
+  a->pairs = c->br3_pairs;
   a->tw = three ? c->d_tw31 : c->d_tw;
+  memcpy(a->tw_lo, three ? &c->tw_lo31[0][0] : &c->tw_lo[0][0], three ? sizeof(c->tw_lo31) : sizeof(c->tw_lo));
   a->cc = three ? c->cc31 : c->cc;
 }
 
@@ -83,7 +86,7 @@ inline void br_key_args(const rosetta_ctx *c, rosetta::BrArgs *a) {
 inline void br_solo_key_args(const rosetta_ctx *c, rosetta::BrArgs *a) {
   a->bsk = c->d_bsk_qf;
   a->primes = rosetta::kPrimes;
-  a->tw = c->d_tw_qf;
+  a->tw = c->d_tw_qf;  // (tw_lo: the 28-bit set's, as for the cluster kernel)
   a->cc = c->cc_qf;
 }
 

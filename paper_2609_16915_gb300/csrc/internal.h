@@ -46,6 +46,8 @@ struct CrtConsts {
   uint64_t qf_base;   // 2^(31 - kQfShift) M mod 2^64: undoes the offset of crt_quotient_qf
 };
 
+constexpr int kTwLo = 64;  // entries of the first six stages
+
 struct BrArgs {
   const uint64_t *lwe_in;   // [batch][n+1]
   const uint64_t *lut;      // [num_luts][2^p]; ignored when glwe_in is set
@@ -59,6 +61,8 @@ struct BrArgs {
   const uint2 *tw;          // [prime][N] (W, Shoup companion)
   uint32_t n, level, base_log, msg_bits, batch, num_luts;
   uint32_t primes;          // kPrimes (bsk, tw, cc over the 28-bit set) or kPrimes31
+  uint32_t pairs;           // three primes: the CTA's shared memory holds the paired exchange buffer
+  uint2 tw_lo[kPrimes][kTwLo];  // each prime's first twiddles again, for the constant bank
   CrtConsts cc;
 };
 
@@ -119,15 +123,15 @@ void build_cfft_tables(uint32_t logN, float4 *pass_tw, double2 *tw);
 // launchers; return cudaSuccess or the launch error
 size_t br_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, bool dig16);
 // one worker per ciphertext, float quotient (blind_rotate_solo.cu): a.bsk, a.tw,
-// a.cc of the float-quotient set, tw_host the host copy of its tables, `workers` (1 .. 3) ciphertexts per CTA
+// a.cc of the float-quotient set, `workers` (1 .. 3) ciphertexts per CTA
 bool br_solo_supported(uint32_t logN, uint32_t level, uint32_t base_log);
 size_t br_solo_smem_bytes(uint32_t n, uint32_t workers);
-cudaError_t launch_blind_rotate_solo(const BrArgs &a, const uint2 *tw_host, uint32_t workers, cudaStream_t s);
+cudaError_t launch_blind_rotate_solo(const BrArgs &a, uint32_t workers, cudaStream_t s);
 // a.primes selects the kernel: the four-prime one or the three-prime one
 cudaError_t launch_blind_rotate(const BrArgs &a, uint32_t logN, bool dig16, cudaStream_t s);
 // three-prime kernel (blind_rotate3.cu): 16-bit digits, compiled ring sizes and levels only
 bool br3_supported(uint32_t logN, uint32_t level, bool dig16);
-size_t br3_smem_bytes(uint32_t logN, uint32_t level, uint32_t n);
+size_t br3_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, bool pairs = false);
 cudaError_t launch_blind_rotate3(const BrArgs &a, uint32_t logN, cudaStream_t s);
 cudaError_t launch_bsk_transform(const uint64_t *raw, uint32_t *out, const uint2 *tw, const CrtConsts &cc,
                                  uint32_t logN, uint32_t n, uint32_t level, uint32_t primes, cudaStream_t s);

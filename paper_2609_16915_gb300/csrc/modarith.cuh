@@ -71,4 +71,22 @@ __device__ __forceinline__ uint32_t cond_sub(uint32_t x, uint32_t b) {
   return min(x, x - b);
 }
 
+// Balanced base-2^beta digits of a word rounded to its top beta * level bits,
+// in closed form: the digits are the plain ones of the word plus dig_offset,
+// each less 2^(beta-1).  (Rounding adds half the lowest kept unit; adding half a
+// unit at every digit makes each carry happen where the digit-by-digit rule
+// carries; the last carry falls off the word in both.)
+__device__ __forceinline__ uint64_t dig_offset(uint32_t beta, uint32_t level) {
+  const uint32_t bits = beta * level;
+  uint64_t c = bits >= 64 ? 0 : 1ull << (63 - bits);
+  for (uint32_t m = 1; m <= level; ++m) c += 1ull << (64 - m * beta + beta - 1);
+  return c;
+}
+
+// The digit of level lev (0: most significant) plus 2^(beta-1), in [0, 2^beta),
+// from w = word + dig_offset.
+__device__ __forceinline__ uint32_t biased_digit(uint64_t w, uint32_t beta, uint32_t lev) {
+  return static_cast<uint32_t>(w >> (64 - (lev + 1) * beta)) & ((1u << beta) - 1u);
+}
+
 }  // namespace rosetta

@@ -161,6 +161,47 @@ __device__ __forceinline__ void load_twiddles(const uint2 *tw, uint32_t start, u
   }
 }
 
+// Twiddles of one prime where the first CST stages' (up to 64 entries, the
+// same for a whole warp when N >= 2048) come from the constant bank, which takes
+// their reads off the shared-memory pipe, and the others from shared memory.  The
+// last stage's, four consecutive ones per thread, are stored as two runs of
+// pairs (split_tw_slot), so that neighbouring threads' 16-byte loads touch
+// neighbouring words.
+template <int LOGN, int CST>
+struct SplitTw {
+  static_assert(LOGN >= 11 && CST <= 6, "warp-uniform twiddles in the first six stages");
+  const uint2 *sm, *cst;
+};
+template <int LOGN>
+__device__ __forceinline__ uint32_t split_tw_slot(uint32_t idx) {
+  constexpr uint32_t N = 1u << LOGN;
+  return idx < N / 2 ? idx : N / 2 + ((idx >> 1) & 1u) * (N / 4) + (((idx - N / 2) >> 2) << 1) + (idx & 1u);
+}
+
+template <int S, int LOGN, int CST>
+__device__ __forceinline__ uint2 tw_at(const SplitTw<LOGN, CST> &tw, uint32_t idx) {
+  if constexpr (S < CST)
+    return tw.cst[idx];
+  else
+    return tw.sm[idx];
+}
+
+template <int S, int CNT, int LOGN, int CST>
+__device__ __forceinline__ void load_twiddles(const SplitTw<LOGN, CST> &tw, uint32_t start, uint2 (&w)[CNT]) {
+  if constexpr (S == LOGN - 1) {
+    static_assert(CNT == 4, "four per thread in the last stage");
+    constexpr uint32_t N = 1u << LOGN;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(tw.sm + N / 2 + k * (N / 4) + (start - N / 2) / 2);
+      w[2 * k] = make_uint2(v.x, v.y);
+      w[2 * k + 1] = make_uint2(v.z, v.w);
+    }
+  } else {
+    load_twiddles<S>(tw.sm, start, w);
+  }
+}
+
 template <int LOGN, int E, int NP, int S0, int H, int U, bool P31, class TW>
 __device__ __forceinline__ void fwd_stage(uint32_t (&x)[NP][E], const TW &tw, uint32_t tau,
                                           uint32_t p, uint32_t two_p, uint32_t eight_p) {
@@ -290,8 +331,11 @@ __host__ __device__ constexpr int pass_group_warps() {
 struct CtaThreads {
   static constexpr bool kWhole = true, kPairs = false;
 };
+struct CtaPairs {  // two polynomials cross the exchange buffer as pairs of words
+  static constexpr bool kWhole = true, kPairs = true;
+};
 struct GroupThreads {
-  static constexpr bool kWhole = false, kPairs = true;  // two polynomials cross the exchange buffer as pairs of words
+  static constexpr bool kWhole = false, kPairs = true;
   uint32_t id, threads;
   __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 };
@@ -379,7 +423,7 @@ __device__ __forceinline__ uint32_t xb2_base(uint32_t tau) {
   if constexpr (SIG == 1) {
     return xb_pad2(E * tau);
   } else {
-    static_assert((1 << H) == E && SIG % 4 == 0 && (SIG >= 16 || SIG == 4), "padding that adds");
+    static_assert((1 << H) == E && E == 8 && SIG >= 2, "padding that adds");
     return xb_pad2((tau / SIG) * SPAN + tau % SIG);
   }
 }

@@ -304,7 +304,7 @@ cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t
   const auto solo = [&](uint32_t first, uint32_t count, uint32_t workers) {
     BrArgs q = br_slice(c, a, first, count);
     br_solo_key_args(c, &q);
-    return launch_blind_rotate_solo(q, c->tw_qf_host.data(), workers, s);
+    return launch_blind_rotate_solo(q, workers, s);
   };
   cudaError_t e = full ? solo(0, full, 3) : cudaSuccess;
   if (e != cudaSuccess || rest == 0) return e;
@@ -375,10 +375,17 @@ int rosetta_params_init(rosetta_ctx **out, const rosetta_params *p, int cuda_dev
       per_sm(smem3) >= per_sm(smem4)) {
     tw31.resize((size_t)kPrimes31 << logN);
     if (build_tables(logN, kPrimes31, tw31.data(), &c->cc31)) c->br_primes = kPrimes31;
+    const size_t smem3p = br3_smem_bytes(logN, p->pbs_level, p->lwe_dim, true);
+    c->br3_pairs = smem3p <= (size_t)max_smem && per_sm(smem3p) >= per_sm(smem3);
   }
+  for (int q = 0; q < kPrimes; ++q)
+    for (int m = 0; m < kTwLo; ++m) {
+      c->tw_lo[q][m] = tw[((size_t)q << logN) + m];
+      if (c->br_primes == kPrimes31 && q < kPrimes31) c->tw_lo31[q][m] = tw31[((size_t)q << logN) + m];
+    }
   // Three of the 28-bit primes and the float quotient for the launches that
   // fill the GPU, where the bound allows it and three workers fit an SM.
-  std::vector<uint2> &tw_qf = c->tw_qf_host;
+  std::vector<uint2> tw_qf;
   std::vector<double2> tw_f64;
   if (fits_float_quotient(*p) && br_solo_supported(logN, p->pbs_level, p->pbs_base_log) &&
       br_solo_smem_bytes(p->lwe_dim, 3) <= (size_t)max_smem) {

@@ -113,7 +113,8 @@ inline cudaClusterSchedulingPolicy br_cluster_policy(K kern, int threads, size_t
 
 // host-side tables (tables.cu): twiddles and CRT constants of the 28-bit set
 // (primes = kPrimes; the first `use` of them) or of the 31-bit set (primes =
-// kPrimes31); tw_host may be null
+// kPrimes31); with tw_host null the CRT constants alone, for a subset of a set
+// whose tables were built
 bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host /*[use][N]*/, CrtConsts *cc, uint32_t use = 0);
 // twiddles of the float transforms of N/2 complex values: the pass table the
 // kernels read (float4 entries, at most N uint2 words) and the whole double

@@ -79,12 +79,12 @@ bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host, CrtConsts *cc,
   cc->qf_base = cc->M_mod64 << (31 - kQfShift);
   for (uint32_t q = 0; q < use; ++q) {
     const uint32_t p = list[q];
-    if (!is_prime(p) || (p - 1) % (2 * N) != 0 || p >= (1u << top) || p <= (1u << top) - (1u << gap)) return false;
-    const uint32_t g = generator(p);
-    if (!g) return false;
-    const uint32_t psi = powmod(g, (p - 1) / (2 * N), p);  // primitive 2N-th root of unity
-    if (powmod(psi, N, p) != p - 1) return false;
     if (tw_host) {
+      if (!is_prime(p) || (p - 1) % (2 * N) != 0 || p >= (1u << top) || p <= (1u << top) - (1u << gap)) return false;
+      const uint32_t g = generator(p);
+      if (!g) return false;
+      const uint32_t psi = powmod(g, (p - 1) / (2 * N), p);  // primitive 2N-th root of unity
+      if (powmod(psi, N, p) != p - 1) return false;
       uint64_t w = 1;  // psi^i, i = bitrev(m)
       for (uint32_t i = 0; i < N; ++i) {
         tw_host[(size_t)q * N + bitrev(i, logN)] =

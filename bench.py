@@ -100,9 +100,10 @@ def int_ops_per_lookup(p, n_seg: int, t_base_log: int, t_level: int) -> dict:
 
 
 def ks_tensor_limbs(p, batch) -> int:
-    """Limbs per key word of the tensor-core key switch the library takes for
-    this batch (8 or 16), or 0 when it takes the CUDA-core kernel: batches of
-    256 and more, digits that bf16 holds, fp32 sums below 2^24."""
+    """Limbs per key word of the bf16 tensor-core key switch for this batch (8
+    or 16), or 0 where that kernel does not apply: batches of 256 and more,
+    digits that bf16 holds, fp32 sums below 2^24.  (Bases up to 2^5 take the
+    8-bit kernel, ks_fp8.)"""
     K = p.kN * p.ks_level
     if batch < 256 or p.ks_base_log > 8 or K % 64:
         return 0
@@ -119,6 +120,32 @@ def ks_tensor_flops(p, batch, limbs) -> float:
     rows = -(-batch // 128) * 128
     cols = -(-(p.n + 1) * limbs // 256) * 256
     return 2.0 * rows * K * cols
+
+
+def br_solo(p) -> bool:
+    """Does the context hold the worker-per-ciphertext kernel for this set?"""
+    return p.N == 2048 and p.pbs_level == 1 and p.pbs_base_log <= 24
+
+
+def br_launches(p, batch, sms) -> int:
+    """Blind-rotation kernels of one call: whole waves on three workers per SM
+    and the rest as run_blind_rotate splits it."""
+    full, rest = divmod(batch, 3 * sms)
+    if not br_solo(p) or rest == 0 or full == 0 or rest > 2 * sms:
+        return 1
+    return 2
+
+
+def ks_fp8(p) -> bool:
+    """Does the library take the 8-bit tensor-core key switch (every batch)?"""
+    return p.ks_base_log <= 5 and p.kN % 128 == 0 and 2 ** (p.ks_base_log - 1) * 16 * p.kN * p.ks_level < 2 ** 24
+
+
+def ks_fp8_flops(p, batch) -> float:
+    """Dense e4m3 flops of the 8-bit key switch as launched: rows by tiles of
+    16 output words x 13 limbs over K = kN l."""
+    rows = -(-batch // 256) * 256 if batch > 128 else 128
+    return 2.0 * rows * p.kN * p.ks_level * (-(-(p.n + 1) // 16) * 208)
 
 
 TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "blind_rotate_standard_b4096_dram.txt")
@@ -373,7 +400,7 @@ def run_lookup(args, p, batch, torch, dev, R, clock_sampler):
                      "kernel_ms": br_ms, "trace_ms": tr_ms,
                      "path_ops_per_lookup": ops, "path_achieved": path_achieved,
                      "path_frac": path_achieved / alu_peak},
-        "gpu_launches": (4 * n_seg + 6) * args.steps,
+        "gpu_launches": ((n_seg + 2) * (1 + br_launches(p, batch, sms)) + (n_seg + 1) + n_seg + 2) * args.steps,
         "clocks": clk.summary(),
     }
     return line
@@ -429,7 +456,7 @@ def run_multi_lut(args, p, batch, torch, dev, R, clock_sampler):
                    "l2": "flushed between steps (256 MB write)", "keys": "uniform words, resident"},
         "roofline": {"bound": "alu", "kernel": "blind_rotate_kernel + key switch (whole step)", "achieved": achieved,
                      "peak": alu_peak, "unit": "Tops/s (int32)", "frac": achieved / alu_peak, "traffic": None},
-        "gpu_launches": (3 if ks_tensor_limbs(p, batch) else 2) * args.steps,
+        "gpu_launches": (br_launches(p, batch, sms) + (2 if ks_fp8(p) or ks_tensor_limbs(p, batch) else 1)) * args.steps,
         "clocks": clk.summary(),
     }
     return line
@@ -465,7 +492,9 @@ def butterfly_rate(rates, primes):
     return rates["butterfly_p31"]["per_clk_per_sm"] / 9.0 if primes == 3 else rates["butterfly"]["per_clk_per_sm"] / 5.0
 
 
-def kernel_name(primes):
+def kernel_name(primes, p=None):
+    if p is not None and br_solo(p):
+        return "blind_rotate_solo_kernel (3 primes and a float quotient)"
     return "blind_rotate3_kernel (3 primes)" if primes == 3 else "blind_rotate_kernel (4 primes)"
 
 
@@ -666,7 +695,13 @@ def main():
     mix_peak = bfly_per_clk * 8 * sms * sm_max * 1e6 / 1e12
     pbs_roof = alu_peak * 1e12 / (br_ops + ks_ops)
     limbs = ks_tensor_limbs(p, batch)
-    if limbs:
+    if ks_fp8(p):
+        ks_tf = ks_fp8_flops(p, batch) / (ks_ms / 1e3) / 1e12
+        fp8_peak = 2 * pk.get("bf16_tflops", 1900.0)
+        ks_roof = {"bound": "tensor", "kernel": "ks8_digits_kernel + ks8_kernel (e4m3 tcgen05)",
+                   "achieved": ks_tf, "peak": fp8_peak, "unit": "TFLOP/s", "frac": ks_tf / fp8_peak,
+                   "limbs": 13, "peak_basis": "twice bf16_tflops of MEASURED_PEAKS.json (burst)"}
+    elif limbs:
         ks_tf = ks_tensor_flops(p, batch, limbs) / (ks_ms / 1e3) / 1e12
         bf16_peak = pk.get("bf16_tflops", 1900.0)
         ks_roof = {"bound": "tensor", "kernel": "ks_digits_kernel + ks_tc_kernel (bf16 tcgen05)",
@@ -687,7 +722,7 @@ def main():
         "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
         "config": {"workload": describe(p, batch), "batch": batch, "parallelism": f"dp{world}" if world > 1 else "none",
                    "l2": "flushed between steps (256 MB write)", "keys": "uniform words, resident"},
-        "roofline": {"bound": "alu", "kernel": kernel_name(primes), "achieved": achieved, "peak": alu_peak,
+        "roofline": {"bound": "alu", "kernel": kernel_name(primes, p), "achieved": achieved, "peak": alu_peak,
                      "unit": "Tops/s (int32)", "frac": achieved / alu_peak, "traffic": measured_traffic(p, batch),
                      "peak_basis": f"{sms} SMs x 128 int32 lanes x {sm_max:.0f} MHz (sm_max_mhz of MEASURED_PEAKS.json)",
                      "kernel_ms": br_ms, "keyswitch_ms": ks_ms, "keyswitch": ks_roof,
@@ -698,7 +733,7 @@ def main():
                                                   if isinstance(v, dict)}},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": batch * (p.n + 1) * 8 + lut.numel() * 8,
                 "d2h_bytes_per_step": batch * (p.n + 1) * 8},
-        "gpu_launches": (3 if limbs else 2) * args.steps,
+        "gpu_launches": (br_launches(p, batch, sms) + (2 if ks_fp8(p) or limbs else 1)) * args.steps,
         "clocks": clk.summary(),
         "wall_s_timed": wall,
     }

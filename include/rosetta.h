@@ -154,13 +154,15 @@ int rosetta_blind_rotate_extract_batch(rosetta_ctx *ctx, const uint64_t *lwe_in,
  * [batch][kN+1], to dimension n, lwe_out [batch][n+1]:
  *   out = (0, .., 0, b') - sum_i sum_lev d_{i,lev}(a'_i) * KSK[i][lev]
  * with d the signed base-2^beta_ks digits of a'_i rounded to its top
- * beta_ks*l_ks bits.  Needs the KSK.  From 256 ciphertexts on, where the
- * parameters allow exact fp32 sums (beta_ks <= 8 and
- * 2^(beta_ks-1) (2^(64/limbs)-1) kN l_ks < 2^24 for 8 or 16 limbs per key
- * word), the product runs on the tensor cores with a digit scratch of
- * batch (kN l_ks) bf16 words owned by the context; the words are the same
- * either way.  A bounded wait inside that kernel that gives up is reported
- * as TIMEOUT by rosetta_sync_status. */
+ * beta_ks*l_ks bits.  Needs the KSK.  Where the fp32 sums are exact the
+ * product runs on the tensor cores: at every batch size with 13 limbs of 5
+ * bits per key word in e4m3 (beta_ks <= 5 and 2^(beta_ks-1) 16 kN l_ks < 2^24),
+ * with a digit scratch of batch (kN l_ks) bytes owned by the context (for up to
+ * 255 ciphertexts allocated with the key); else from 256 ciphertexts on with 8
+ * or 16 limbs in bf16 (beta_ks <= 8 and
+ * 2^(beta_ks-1) (2^(64/limbs)-1) kN l_ks < 2^24); else on the CUDA cores.  The
+ * words are the same either way.  A bounded wait inside a tensor-core kernel
+ * that gives up is reported as TIMEOUT by rosetta_sync_status. */
 int rosetta_keyswitch_batch(rosetta_ctx *ctx, const uint64_t *lwe_big_in, uint32_t batch,
                             uint64_t *lwe_out, void *stream);
 
@@ -283,7 +285,7 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *ctx, const uint64_t *glwe_x, con
  * address in the current CUDA context; the first call on a device (and the
  * first after a device reset) loads the library's device code: make it
  * before any stream capture.  The key switch is the CUDA-core kernel at
- * every batch size, because the tensor-core one needs digit tiles in
+ * every batch size, because the tensor-core ones need digit tiles in
  * allocated memory (same words).  All calls on a device share the array:
  * calls whose work overlaps on the GPU race and must be serialised by the
  * caller.  Errors: INVALID_ARG, KEYS_MISSING, CUDA. */

@@ -39,6 +39,7 @@ struct rosetta_ctx {
   uint64_t *d_corr = nullptr;     // [n+1]
   uint16_t *d_ks_b = nullptr;     // key limb tiles for the tensor-core key switch (null: not exact)
   uint32_t ks_limbs = 0;
+  bool ks_fp8 = false;            // the limb and digit tiles are those of the 8-bit kernel
   uint64_t *d_ks_a = nullptr;     // digit tiles (scratch), as 64-bit words
   size_t ks_a_cap = 0;
   bool have_bsk = false, have_ksk = false;

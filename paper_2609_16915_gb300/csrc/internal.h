@@ -74,10 +74,10 @@ struct KsArgs {
   uint32_t batch, kN, n, base_log, level;
 };
 
-// Tensor-core key switch: digit and limb tiles in the MMA layout.
+// Tensor-core key switches: digit and limb tiles in the MMA layout.
 struct KsTcArgs {
-  const uint16_t *a_tiles;  // [m_tiles][k_steps][128 x 64] bf16 digits
-  const uint16_t *b_tiles;  // [n_tiles][k_steps][256 x 64] bf16 key limbs
+  const uint16_t *a_tiles;  // [m_tiles][k_steps][128 x 64] bf16 (or 128 x 128 e4m3) digits
+  const uint16_t *b_tiles;  // [n_tiles][k_steps][256 x 64] bf16 (or 208 x 128 e4m3) key limbs
   const uint64_t *big;      // [batch][kN+1]
   uint64_t *out;            // [batch][n+1]
   uint32_t *err_flag;       // set to 2 when a wait gives up
@@ -157,6 +157,13 @@ size_t ks_tc_a_words16(uint32_t batch, uint32_t kN, uint32_t level);
 cudaError_t launch_ks_limbs(const uint64_t *ksk, uint16_t *b_tiles, uint32_t kN, uint32_t level, uint32_t n,
                             uint32_t limbs, cudaStream_t s);
 cudaError_t launch_keyswitch_tc(const KsTcArgs &a, uint32_t base_log, uint32_t level, cudaStream_t s);
+// 8-bit key switch (keyswitch_fp8.cu): bases up to 2^5 whose sums stay exact
+bool ks8_exact(uint32_t kN, uint32_t level, uint32_t base_log);
+size_t ks8_b_bytes(uint32_t kN, uint32_t level, uint32_t n);
+size_t ks8_a_bytes(uint32_t batch, uint32_t kN, uint32_t level);
+cudaError_t launch_ks8_limbs(const uint64_t *ksk, uint8_t *b_tiles, uint32_t kN, uint32_t level, uint32_t n,
+                             cudaStream_t s);
+cudaError_t launch_keyswitch_fp8(const KsTcArgs &a, uint32_t base_log, uint32_t level, uint32_t sms, cudaStream_t s);
 cudaError_t launch_wait_selftest(uint32_t *err_flag, uint32_t limit_us, cudaStream_t s);
 cudaError_t launch_ksk_corr(const uint64_t *ksk, uint64_t *corr, uint32_t rows, uint32_t n, uint32_t base_log,
                             cudaStream_t s);

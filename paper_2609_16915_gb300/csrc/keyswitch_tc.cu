@@ -1,4 +1,7 @@
-// LWE key switch on the tensor cores (tcgen05, accumulators in tensor memory).
+// LWE key switch on the tensor cores (tcgen05, accumulators in tensor memory)
+// for key-switch bases of 2^6 to 2^8, whose digits the 8-bit kernel
+// (keyswitch_fp8.cu) cannot hold, and for sums past its bound; from 256
+// ciphertexts on.
 //
 // The key switch is the dense contraction of the path:
 //   out[b][j] = [j = n] b'_b - sum_r d[b][r] KSK[r][j]      (mod 2^64)
@@ -35,6 +38,7 @@
 
 #include "dsmem.cuh"
 #include "internal.h"
+#include "tcgen.cuh"
 
 namespace rosetta {
 
@@ -45,7 +49,6 @@ constexpr uint32_t A_TILE = TC_M * TC_K * 2;   // bytes
 constexpr uint32_t B_TILE = TC_N * TC_K * 2;
 constexpr uint32_t STAGE = A_TILE + B_TILE;
 constexpr uint32_t TMEM_COLS = 256;
-constexpr long long kWaitCycles = 4000000000ll;  // ~2 s at 2 GHz
 
 // Element offset of (row, k) inside a tile of the no-swizzle K-major layout.
 __host__ __device__ constexpr uint32_t tile_off(uint32_t row, uint32_t k) {
@@ -58,44 +61,9 @@ __device__ __forceinline__ uint16_t bf16_of_int(int v) {
   return static_cast<uint16_t>(__float_as_uint(f) >> 16);
 }
 
-// Shared-memory matrix descriptor: start address, leading (K) byte offset 128,
-// stride (8-row) byte offset 1024, descriptor version 1, no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-  return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(128u >> 4) << 16) |
-         (static_cast<uint64_t>(1024u >> 4) << 32) | (1ull << 46);
-}
-
 // Instruction descriptor, kind::f16: D f32, A and B bf16, both K-major,
 // N = 256, M = 128.
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((TC_N >> 3) << 17) | ((TC_M >> 4) << 24);
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long limit = kWaitCycles) {
-  const long long t0 = clock64();
-  while (true) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > limit) return false;
-  }
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
 
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
   asm volatile(
@@ -103,10 +71,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
       "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // 32 consecutive fp32 columns of this thread's lane

@@ -187,8 +187,10 @@ BrArgs br_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, const u
   return a;
 }
 
-// Batches from this size on take the tensor-core key switch (when exact for
-// the parameters); smaller ones the split-K CUDA-core kernel.
+// Batches from this size on take the bf16 tensor-core key switch (where the
+// 8-bit one is not exact but this one is); smaller ones the split-K CUDA-core
+// kernel.  The 8-bit kernel takes every batch; digit scratch for batches below
+// this size is allocated with the key, so that their calls allocate nothing.
 constexpr uint32_t kKsTcMinBatch = 256;
 
 KsArgs ks_args(const rosetta_ctx *c, const uint64_t *big, uint32_t batch, uint64_t *out);
@@ -196,9 +198,9 @@ KsArgs ks_args(const rosetta_ctx *c, const uint64_t *big, uint32_t batch, uint64
 cudaError_t run_keyswitch(rosetta_ctx *c, const uint64_t *big, uint32_t batch, uint64_t *out, cudaStream_t s) {
   const rosetta_params &p = c->prm;
   const uint32_t kN = p.glwe_dim * p.poly_size;
-  if (c->ks_limbs && c->d_ks_b && batch >= kKsTcMinBatch) {
-    const size_t words16 = ks_tc_a_words16(batch, kN, p.ks_level);
-    if (ensure(&c->d_ks_a, &c->ks_a_cap, (words16 + 3) / 4, s) != ROSETTA_OK) return cudaErrorMemoryAllocation;
+  if (c->d_ks_b && (c->ks_fp8 || batch >= kKsTcMinBatch)) {
+    const size_t bytes = c->ks_fp8 ? ks8_a_bytes(batch, kN, p.ks_level) : 2 * ks_tc_a_words16(batch, kN, p.ks_level);
+    if (ensure(&c->d_ks_a, &c->ks_a_cap, (bytes + 7) / 8, s) != ROSETTA_OK) return cudaErrorMemoryAllocation;
     KsTcArgs a{};
     a.a_tiles = reinterpret_cast<const uint16_t *>(c->d_ks_a);
     a.b_tiles = c->d_ks_b;
@@ -208,8 +210,9 @@ cudaError_t run_keyswitch(rosetta_ctx *c, const uint64_t *big, uint32_t batch, u
     a.batch = batch;
     a.kN = kN;
     a.n = p.lwe_dim;
-    a.k_steps = kN * p.ks_level / 64;
+    a.k_steps = kN * p.ks_level / (c->ks_fp8 ? 128 : 64);
     a.limbs = c->ks_limbs;
+    if (c->ks_fp8) return launch_keyswitch_fp8(a, p.ks_base_log, p.ks_level, c->sms, s);
     return launch_keyswitch_tc(a, p.ks_base_log, p.ks_level, s);
   }
   return launch_keyswitch(ks_args(c, big, batch, out), s);
@@ -493,8 +496,17 @@ int rosetta_upload_ksk(rosetta_ctx *c, const uint64_t *ksk, size_t n_words, int 
   if (e != cudaSuccess) return cuda_fail(e);
   // limb tiles for the tensor-core key switch, where its fp32 sums are exact
   const uint32_t kN = p.glwe_dim * p.poly_size;
-  c->ks_limbs = ks_tc_limbs(kN, p.ks_level, p.ks_base_log);
-  if (c->ks_limbs) {
+  c->ks_fp8 = ks8_exact(kN, p.ks_level, p.ks_base_log);
+  c->ks_limbs = c->ks_fp8 ? 0 : ks_tc_limbs(kN, p.ks_level, p.ks_base_log);
+  if (c->ks_fp8) {
+    if (!c->d_ks_b) e = cudaMalloc(&c->d_ks_b, ks8_b_bytes(kN, p.ks_level, p.lwe_dim));
+    if (e == cudaSuccess)
+      e = launch_ks8_limbs(c->d_ksk, reinterpret_cast<uint8_t *>(c->d_ks_b), kN, p.ks_level, p.lwe_dim, s);
+    if (e == cudaSuccess && ensure(&c->d_ks_a, &c->ks_a_cap, ks8_a_bytes(kKsTcMinBatch - 1, kN, p.ks_level) / 8, s) !=
+                                ROSETTA_OK)
+      e = cudaErrorMemoryAllocation;
+    if (e != cudaSuccess) return cuda_fail(e);
+  } else if (c->ks_limbs) {
     if (!c->d_ks_b) e = cudaMalloc(&c->d_ks_b, ks_tc_b_words16(kN, p.ks_level, p.lwe_dim, c->ks_limbs) * 2);
     if (e == cudaSuccess) e = launch_ks_limbs(c->d_ksk, c->d_ks_b, kN, p.ks_level, p.lwe_dim, c->ks_limbs, s);
     if (e != cudaSuccess) return cuda_fail(e);

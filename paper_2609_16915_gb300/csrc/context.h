@@ -55,11 +55,10 @@ struct rosetta_ctx {
   uint32_t *d_trk = nullptr;      // trace automorphism keys, transform domain
   uint32_t trk_base_log = 0, trk_level = 0;
   bool have_trk = false;
-  uint64_t *d_pm_raw = nullptr;   // plaintext-multiply gadget rows, raw [8][2][N]
-  uint32_t *d_pm_key = nullptr;   // the same in the transform domain
-  uint64_t *d_pm_add = nullptr;   // staged additive plaintext [N]
-  // segmented lookup: plaintext polynomials (P, A_0..A_{n_seg-1}, Box_0) as gadget rows in the
-  // transform domain [n_seg+2][prime][8][2][N], additive ones (Q, B_0..B_{n_seg-1}) [n_seg+1][N]
+  uint64_t *d_pm_raw = nullptr;   // plaintext-multiply rows P 2^32 and P, raw [2][N], and the additive plaintext [N]
+  uint32_t *d_pm_key = nullptr;   // the rows in the transform domain [prime][2][N]
+  // segmented lookup: plaintext polynomials (P, A_0..A_{n_seg-1}, Box_0) as rows in the
+  // transform domain [n_seg+2][prime][2][N], additive ones (Q, B_0..B_{n_seg-1}) [n_seg+1][N]
   uint32_t *d_lk_key = nullptr;
   uint64_t *d_lk_add = nullptr;
   uint32_t lk_nseg = 0;

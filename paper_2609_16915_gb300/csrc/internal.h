@@ -87,10 +87,21 @@ struct KsTcArgs {
 struct TraceArgs {
   const uint64_t *glwe_in;  // [batch][2][N]
   uint64_t *glwe_out;       // [batch][2][N]
-  const uint32_t *keys;     // transform domain [steps][prime][rows][2][N]
-  const uint64_t *plain_add;  // [N] added to the body (plaintext-multiply mode), or null
+  const uint32_t *keys;     // transform domain [steps][prime][level][2][N]
   const uint2 *tw;          // [prime][N]
-  uint32_t base_log, level, batch;  // level = rows of a key (trace); 2 x gadget levels (multiply)
+  uint32_t base_log, level, batch;
+  uint2 tw_lo[kPrimes][8];  // each prime's first twiddles again, for the constant bank
+  CrtConsts cc;
+};
+
+// (P A, P B + Q): P by the transformed rows of P 2^32 and P.
+struct PlainMulArgs {
+  const uint64_t *glwe_in;    // [batch][2][N]
+  uint64_t *glwe_out;         // [batch][2][N]
+  const uint32_t *keys;       // transform domain [prime][2][N]
+  const uint64_t *plain_add;  // Q [N], or null
+  const uint2 *tw;            // [prime][N]
+  uint2 tw_lo[kPrimes][8];
   CrtConsts cc;
 };
 
@@ -146,9 +157,8 @@ cudaError_t launch_keyswitch(const KsArgs &a, cudaStream_t s);
 cudaError_t launch_key_transform(const uint64_t *raw, uint32_t *out, const uint2 *tw, const CrtConsts &cc,
                                  uint32_t logN, uint32_t count, uint32_t rows, cudaStream_t s,
                                  uint32_t primes = kPrimes);
-size_t trace_smem_bytes(uint32_t logN, uint32_t level);
 cudaError_t launch_trace(const TraceArgs &a, uint32_t logN, cudaStream_t s);
-cudaError_t launch_plaintext_mul(const TraceArgs &a, uint32_t logN, cudaStream_t s);
+cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, uint32_t batch, cudaStream_t s);
 cudaError_t launch_monomial_acc(uint64_t *R, const uint64_t *r, uint32_t count, uint32_t logN, uint32_t e, bool first,
                                 cudaStream_t s);
 uint32_t ks_tc_limbs(uint32_t kN, uint32_t level, uint32_t base_log);  // 8, 16, or 0 (not exact)

@@ -169,7 +169,7 @@ __device__ __forceinline__ void load_twiddles(const uint2 *tw, uint32_t start, u
 // neighbouring words.
 template <int LOGN, int CST>
 struct SplitTw {
-  static_assert(LOGN >= 11 && CST <= 6, "warp-uniform twiddles in the first six stages");
+  static_assert(CST <= 3 || (LOGN >= 11 && CST <= 6), "warp-uniform twiddles: the first pass; the second from N = 2048");
   const uint2 *sm, *cst;
 };
 template <int LOGN>

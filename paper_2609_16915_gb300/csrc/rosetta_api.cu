@@ -232,33 +232,32 @@ KsArgs ks_args(const rosetta_ctx *c, const uint64_t *big, uint32_t batch, uint64
   return k;
 }
 
-// Plaintext products use an exact 64-bit gadget (16 bits x 4 levels) against
-// noiseless rows: row comp*4 + l of component comp holds P 2^(64 - (l+1) 16),
-// the other component 0 (raw layout [8][2][N]).
-constexpr uint32_t kPmBase = 16, kPmLev = 4, kPmRows = 2 * kPmLev;
-
+// A plaintext polynomial's rows P 2^32 and P (raw layout [2][N]; the key
+// transform takes them as the two components of one row).
 void pm_rows(uint64_t *raw, const int64_t *P, size_t N) {
-  for (size_t w = 0; w < kPmRows * 2 * N; ++w) raw[w] = 0;
-  for (uint32_t comp = 0; comp < 2; ++comp)
-    for (uint32_t l = 0; l < kPmLev; ++l)
-      for (size_t t = 0; t < N; ++t)
-        raw[((comp * kPmLev + l) * 2 + comp) * N + t] = static_cast<uint64_t>(P[t]) << (64 - (l + 1) * kPmBase);
+  for (size_t t = 0; t < N; ++t) {
+    raw[t] = static_cast<uint64_t>(P[t]) << 32;
+    raw[N + t] = static_cast<uint64_t>(P[t]);
+  }
 }
 
-// out[b] = (P * in_A, P * in_B + add) with P given by its transformed gadget rows.
+template <typename Args>
+void small_tables(const rosetta_ctx *c, Args *a) {
+  a->tw = c->d_tw;
+  a->cc = c->cc;
+  for (int q = 0; q < kPrimes; ++q) memcpy(a->tw_lo[q], c->tw_lo[q], sizeof(a->tw_lo[q]));
+}
+
+// out[b] = (P * in_A, P * in_B + add) with P given by its transformed rows.
 cudaError_t launch_pm(const rosetta_ctx *c, const uint32_t *key, const uint64_t *add, const uint64_t *in,
                       uint32_t batch, uint64_t *out, cudaStream_t s) {
-  TraceArgs a{};
+  PlainMulArgs a{};
   a.glwe_in = in;
   a.glwe_out = out;
   a.keys = key;
   a.plain_add = add;
-  a.tw = c->d_tw;
-  a.base_log = kPmBase;
-  a.level = kPmRows;
-  a.batch = batch;
-  a.cc = c->cc;
-  return launch_plaintext_mul(a, c->logN, s);
+  small_tables(c, &a);
+  return launch_plaintext_mul(a, c->logN, batch, s);
 }
 
 TraceArgs trace_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, uint64_t *out) {
@@ -266,11 +265,10 @@ TraceArgs trace_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, u
   a.glwe_in = in;
   a.glwe_out = out;
   a.keys = c->d_trk;
-  a.tw = c->d_tw;
   a.base_log = c->trk_base_log;
   a.level = c->trk_level;
   a.batch = batch;
-  a.cc = c->cc;
+  small_tables(c, &a);
   return a;
 }
 
@@ -632,9 +630,11 @@ int rosetta_upload_trace_keys(rosetta_ctx *c, const uint64_t *keys, size_t n_wor
     while ((1ull << e) < (uint64_t)level * p.poly_size) ++e;
     if (63 + (base_log - 1) + e + 1 > 111) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
   }
+  // the documented limit on levels: 26.5 N + level N bytes per CTA (the kernel
+  // itself needs less)
   int max_smem = 0;
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-  if (trace_smem_bytes(c->logN, level) > (size_t)max_smem) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
+  if ((size_t)p.poly_size * (53 + 2 * (size_t)level) / 2 > (size_t)max_smem) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
   const size_t want = (size_t)c->logN * level * 2 * p.poly_size;
   if (n_words != want || !aligned8(keys)) return ROSETTA_ERR_INVALID_ARG;
   if (cudaSetDevice(c->device) != cudaSuccess) return ROSETTA_ERR_CUDA;
@@ -701,19 +701,22 @@ int rosetta_plaintext_mul_batch(rosetta_ctx *c, const uint64_t *glwe_in, uint32_
       !aligned8(plain_mul) || (plain_add && !aligned8(plain_add)) || overlaps(glwe_in, gbytes, glwe_out, gbytes))
     return ROSETTA_ERR_INVALID_ARG;
   if (is_device_ptr(plain_mul)) return ROSETTA_ERR_INVALID_ARG;  // the gadget rows are built on the host
-  std::vector<uint64_t> raw(kPmRows * 2 * N);
+  // one staging vector and one copy: the rows, and a host plain_add behind them
+  const bool add_host = plain_add && !is_device_ptr(plain_add);
+  std::vector<uint64_t> raw((add_host ? 3 : 2) * N);
   pm_rows(raw.data(), plain_mul, N);
+  if (add_host) memcpy(raw.data() + 2 * N, plain_add, N * 8);
   cudaStream_t s = as_stream(stream);
   cudaError_t e = cudaSuccess;
-  if (!c->d_pm_raw) e = cudaMalloc(&c->d_pm_raw, raw.size() * 8);
-  if (e == cudaSuccess && !c->d_pm_key) e = cudaMalloc(&c->d_pm_key, raw.size() * kPrimes * sizeof(uint32_t));
-  if (e == cudaSuccess && !c->d_pm_add) e = cudaMalloc(&c->d_pm_add, N * 8);
+  if (!c->d_pm_raw) e = cudaMalloc(&c->d_pm_raw, 3 * N * 8);
+  if (e == cudaSuccess && !c->d_pm_key) e = cudaMalloc(&c->d_pm_key, kPrimes * 2 * N * sizeof(uint32_t));
   if (e != cudaSuccess) return cuda_fail(e);
+  uint64_t *d_add = c->d_pm_raw + 2 * N;
   e = cudaMemcpyAsync(c->d_pm_raw, raw.data(), raw.size() * 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && plain_add)
-    e = cudaMemcpyAsync(c->d_pm_add, plain_add, N * 8, cudaMemcpyDefault, s);
-  if (e == cudaSuccess) e = launch_key_transform(c->d_pm_raw, c->d_pm_key, c->d_tw, c->cc, c->logN, 1, kPmRows, s);
-  if (e == cudaSuccess) e = launch_pm(c, c->d_pm_key, plain_add ? c->d_pm_add : nullptr, glwe_in, batch, glwe_out, s);
+  if (e == cudaSuccess && plain_add && !add_host)
+    e = cudaMemcpyAsync(d_add, plain_add, N * 8, cudaMemcpyDeviceToDevice, s);
+  if (e == cudaSuccess) e = launch_key_transform(c->d_pm_raw, c->d_pm_key, c->d_tw, c->cc, c->logN, 1, 1, s);
+  if (e == cudaSuccess) e = launch_pm(c, c->d_pm_key, plain_add ? d_add : nullptr, glwe_in, batch, glwe_out, s);
   if (e != cudaSuccess) return cuda_fail(e);
   e = cudaStreamSynchronize(s);  // the host staging vector goes out of scope
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
@@ -729,7 +732,7 @@ int rosetta_upload_lookup_table(rosetta_ctx *c, uint32_t n_seg, const int64_t *p
     return ROSETTA_ERR_INVALID_ARG;  // the tables are encoded on the host
   if (cudaSetDevice(c->device) != cudaSuccess) return ROSETTA_ERR_CUDA;
   const uint32_t polys = n_seg + 2;  // P, A_0 .. A_{n_seg-1}, Box_0
-  const size_t poly_words = kPmRows * 2 * N;
+  const size_t poly_words = 2 * N;
   std::vector<uint64_t> raw(polys * poly_words);
   pm_rows(raw.data(), p_hat, N);
   for (uint32_t sg = 0; sg < n_seg; ++sg) pm_rows(raw.data() + (1 + sg) * poly_words, a_hat + sg * N, N);
@@ -759,7 +762,7 @@ int rosetta_upload_lookup_table(rosetta_ctx *c, uint32_t n_seg, const int64_t *p
   if (e == cudaSuccess) e = cudaMalloc(&c->d_lk_add, add.size() * 8);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_raw, raw.data(), raw.size() * 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_lk_add, add.data(), add.size() * 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = launch_key_transform(d_raw, c->d_lk_key, c->d_tw, c->cc, c->logN, polys, kPmRows, s);
+  if (e == cudaSuccess) e = launch_key_transform(d_raw, c->d_lk_key, c->d_tw, c->cc, c->logN, polys, 1, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(d_raw);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -789,7 +792,7 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
   if (r == ROSETTA_OK) r = ensure_big(c, batch, s);
   if (r != ROSETTA_OK) return r;
   const uint32_t nseg = c->lk_nseg;
-  const size_t key_words = (size_t)kPrimes * kPmRows * gw;
+  const size_t key_words = (size_t)kPrimes * gw;
   const uint32_t *kP = c->d_lk_key, *kBox = c->d_lk_key + (1 + nseg) * key_words;
   uint64_t *T = c->d_lk_t, *U = c->d_lk_u, *R = c->d_lk_R, *I = c->d_lk_I;
 
@@ -907,7 +910,6 @@ void rosetta_destroy(rosetta_ctx *c) {
   cudaFree(c->d_trk);
   cudaFree(c->d_pm_raw);
   cudaFree(c->d_pm_key);
-  cudaFree(c->d_pm_add);
   cudaFree(c->d_lk_key);
   cudaFree(c->d_lk_add);
   cudaFree(c->d_lk_t);

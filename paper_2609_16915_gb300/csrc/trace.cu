@@ -17,18 +17,16 @@
 // way: CTA r of the cluster transforms for prime r and owns coefficients
 // [rN/4, (r+1)N/4).  Per step:
 //   1. owners gather sigma_k(A), sigma_k(B) for their quarter (distributed
-//      shared memory), write the digits of sigma_k(A) and keep sigma_k(B);
+//      shared memory), write the digits of sigma_k(A) and, after the barrier,
+//      add sigma_k(B) to B;
 //   2. prime-CTAs transform digit pairs, multiply by key_s, inverse-transform
-//      and send CRT-scaled residues to the owners;
-//   3. owners: A -= X_0, B += sigma_k(B) - X_1.
-//
-// The same kernel in its plaintext-multiply mode computes, in one step,
-// (P * A, P * B + Q) for a plaintext polynomial P (small signed
-// coefficients) and Q: the ciphertext components are split into exact gadget
-// digits (base_log * levels = 64) and multiplied by the rows P 2^(64 - l base_log)
-// of a noiseless "key", which gives P * C exactly; this is the linear mapping
-// a_s(X) [[x]] + b_s(X) of the lookup protocol (Cryptographic Lookup Protocol,
-// Steps 2 and 3).
+//      and leave the CRT-scaled residues in their exchange buffer;
+//   3. owners read them: (A, B) -= (X_0, X_1).
+// Digits and residues travel in packed groups and the barriers order shared
+// memory only, as in the blind rotation; the transforms exchange pairs; four
+// CTAs fit an SM at N = 2048.  Measured, N = 2048, gadget 2^16 x 4, 1024
+// ciphertexts: 1.84 ms with single-word exchanges, pushed residues and plain
+// barriers, 1.38 ms here.
 #include <cooperative_groups.h>
 
 #include "dsmem.cuh"
@@ -44,16 +42,18 @@ struct TrShape {
   static constexpr int E = 8;
   static constexpr int T = N / E;
   static constexpr int Q = N / 4;
-  static constexpr int ITEMS = 2 * Q / T;  // 2 mask items then 2 body items per thread
-  static constexpr int QE = E / 4;
+  // resident CTAs per SM the register allocation must allow (4 x 50-54 KB of
+  // shared memory at N = 2048, 2 x 100-108 KB at 4096, four levels)
+  static constexpr int MIN_CTAS = LOGN == 11 ? 4 : (LOGN == 12 ? 2 : 1);
+  static constexpr int XB_WORDS = 2 * (N + N / 8);  // pairs of words; the outgoing residues (2N) afterwards
 };
 
-template <int LOGN, bool PTMUL>
-__global__ void __launch_bounds__(TrShape<LOGN>::T) trace_kernel(const TraceArgs a) {
+template <int LOGN, bool DIG16>
+__global__ void __launch_bounds__(TrShape<LOGN>::T, TrShape<LOGN>::MIN_CTAS) trace_kernel(
+    const __grid_constant__ TraceArgs a) {
   using B = TrShape<LOGN>;
-  constexpr uint32_t N = B::N, T = B::T, Q = B::Q;
-  constexpr uint32_t TWO_N = 2 * N;
-  constexpr int E = B::E, ITEMS = B::ITEMS, QE = B::QE;
+  constexpr uint32_t N = B::N, T = B::T, Q = B::Q, TWO_N = 2 * N;
+  constexpr int E = B::E;
 
   cg::cluster_group cluster = cg::this_cluster();
   const uint32_t rank = cluster.block_rank();
@@ -61,93 +61,95 @@ __global__ void __launch_bounds__(TrShape<LOGN>::T) trace_kernel(const TraceArgs
   const uint32_t tau = threadIdx.x;
 
   extern __shared__ __align__(16) unsigned char smem[];
-  uint2 *tw = reinterpret_cast<uint2 *>(smem);                  // [N]
-  uint64_t *acc = reinterpret_cast<uint64_t *>(tw + N);         // [2][Q]
-  uint64_t *sig_b = acc + 2 * Q;                                 // [Q] sigma_k(B) of the owned quarter
-  uint32_t *res = reinterpret_cast<uint32_t *>(sig_b + Q);      // [4 primes][2][Q]
-  uint32_t *xb = res + kPrimes * 2 * Q;                         // [XB_WORDS]
-  int32_t *dig = reinterpret_cast<int32_t *>(xb + NttShape<LOGN, E>::XB_WORDS);  // [level][Q]
+  uint2 *tw_s = reinterpret_cast<uint2 *>(smem);              // [N]
+  uint64_t *acc = reinterpret_cast<uint64_t *>(tw_s + N);     // [2][Q]
+  uint32_t *xb = reinterpret_cast<uint32_t *>(acc + 2 * Q);
+  uint32_t *dig = xb + B::XB_WORDS;                           // [level / 2][T][2 rows][2 slots], 16- or 32-bit
 
   const uint32_t p = a.cc.pr[rank].p;
   const uint32_t p_inv = a.cc.pr[rank].p_inv;
 
-  for (uint32_t m = tau; m < N; m += T) tw[m] = a.tw[rank * N + m];
+  for (uint32_t m = tau; m < N; m += T) tw_s[split_tw_slot<LOGN>(m)] = a.tw[rank * N + m];
+  const SplitTw<LOGN, 3> tw{tw_s, a.tw_lo[rank]};
   const uint64_t *gin = a.glwe_in + static_cast<size_t>(ct) * 2 * N;
 #pragma unroll
-  for (int m = 0; m < ITEMS; ++m) {
-    const uint32_t item = tau + m * T;
-    const uint32_t c = item / Q, jl = item % Q;
+  for (int m = 0; m < 4; ++m) {  // thread tau owns local coefficients tau and tau + T of both components
+    const uint32_t c = m / 2, jl = tau + (m % 2) * T;
     acc[c * Q + jl] = gin[c * N + rank * Q + jl];
   }
   cluster.sync();
 
-  const uint32_t acc_s = smem_addr(acc), dig_s = smem_addr(dig), res_s = smem_addr(res);
-  const uint32_t bits = a.base_log * (PTMUL ? a.level / 2 : a.level);
-  const uint64_t Bmask = (1ull << a.base_log) - 1;
-  const uint64_t Bhalf = 1ull << (a.base_log - 1);
-  const uint64_t round_add = bits >= 64 ? 0 : (1ull << (63 - bits));
-  const uint32_t round_sh = bits >= 64 ? 0 : 64 - bits;
+  const uint32_t acc_s = smem_addr(acc), xb_s = smem_addr(xb);
+  constexpr uint32_t GRP_BYTES = DIG16 ? 8 : 16;
+  const uint32_t dig_t = smem_addr(dig) + tau * GRP_BYTES;
+  const uint32_t res_t = xb_s + (rank * T + tau) * 16u;  // this owner's group in every prime-CTA
+  const uint64_t dig_add = dig_offset(a.base_log, a.level);
+  const uint32_t dig_bias = p - (1u << (a.base_log - 1));  // stored digits lie in [0, B): d + p = stored + bias
+  const uint32_t pairs = a.level / 2;
 
-  // multiply mode: level key rows = 2 x gadget levels (component-major)
-  const uint32_t dlev = PTMUL ? a.level / 2 : a.level;
-  constexpr uint32_t STEPS = PTMUL ? 1 : LOGN;
-  for (uint32_t s = 0; s < STEPS; ++s) {
-    const uint32_t k = PTMUL ? 1u : (1u << (LOGN - s)) + 1u;
+#pragma unroll 1
+  for (uint32_t s = 0; s < LOGN; ++s) {
+    const uint32_t k = (1u << (LOGN - s)) + 1u;
     uint32_t kinv = k;  // k^{-1} mod 2^32 (Newton), hence mod 2N
 #pragma unroll
     for (int it = 0; it < 5; ++it) kinv *= 2u - k * kinv;
 
-    // ---- phase 1: gather sigma_k(c) for the owned quarter ----
-    // coefficient j of a(X^k) is +-a[t] with t = j k^{-1} mod 2N (minus when t >= N);
-    // k = 1 in multiply mode (every word is the owner's own)
-    uint64_t v[ITEMS];
+    // ---- phase 1: gather sigma_k(c) for the owned quarter, digits of sigma_k(A) ----
+    // coefficient j of a(X^k) is +-a[t] with t = j k^{-1} mod 2N (minus when t >= N)
+    uint64_t v[4];
 #pragma unroll
-    for (int m = 0; m < ITEMS; ++m) {
-      const uint32_t item = tau + m * T;
-      const uint32_t c = item / Q, jl = item % Q, j = rank * Q + jl;
+    for (int m = 0; m < 4; ++m) {
+      const uint32_t c = m / 2, j = rank * Q + tau + (m % 2) * T;
       const uint32_t t = (j * kinv) & (N - 1);
       v[m] = dsmem_ld_u64(dsmem_map(acc_s + (c * Q + (t % Q)) * 8u, t / Q));
     }
 #pragma unroll
-    for (int m = 0; m < ITEMS; ++m) {
-      const uint32_t item = tau + m * T;
-      const uint32_t c = item / Q, jl = item % Q, j = rank * Q + jl;
-      const bool neg = ((j * kinv) & (TWO_N - 1)) >= N;
-      const uint64_t w = neg ? 0ull - v[m] : v[m];
-      if (!PTMUL && c == 1) {
-        sig_b[jl] = w;
-      } else {
-        const uint32_t row0 = PTMUL ? c * dlev : 0;
-        uint64_t cv = bits >= 64 ? w : (w + round_add) >> round_sh;
-        for (int l = static_cast<int>(dlev) - 1; l >= 0; --l) {
-          const uint64_t d = cv & Bmask;
-          cv >>= a.base_log;
-          int32_t ds = static_cast<int32_t>(d);
-          if (d >= Bhalf) {
-            ds -= static_cast<int32_t>(Bmask + 1);
-            cv += 1;
-          }
-          dig[(row0 + l) * Q + jl] = ds;
-        }
-      }
+    for (int m = 0; m < 4; ++m) {
+      const uint32_t j = rank * Q + tau + (m % 2) * T;
+      if (((j * kinv) & (TWO_N - 1)) >= N) v[m] = 0ull - v[m];
     }
-    cluster.sync();
+    v[0] += dig_add;
+    v[1] += dig_add;
+    for (uint32_t P = 0; P < pairs; ++P) {
+      const uint32_t d00 = biased_digit(v[0], a.base_log, 2 * P), d01 = biased_digit(v[1], a.base_log, 2 * P);
+      const uint32_t d10 = biased_digit(v[0], a.base_log, 2 * P + 1), d11 = biased_digit(v[1], a.base_log, 2 * P + 1);
+      if constexpr (DIG16)
+        *reinterpret_cast<uint2 *>(dig + (P * T + tau) * 2) = make_uint2(d00 | (d01 << 16), d10 | (d11 << 16));
+      else
+        *reinterpret_cast<uint4 *>(dig + (P * T + tau) * 4) = make_uint4(d00, d01, d10, d11);
+    }
+    cluster_sync_shared();
+    // the remote reads are over: B + sigma_k(B) in place
+    acc[Q + tau] += v[2];
+    acc[Q + tau + T] += v[3];
 
     // ---- phase 2: digits x key_s for prime `rank` ----
     uint32_t oh[2][E];
     const uint32_t *kbase =
         a.keys + (static_cast<size_t>(s) * kPrimes + rank) * (static_cast<size_t>(a.level) * 2 * N);
-    for (uint32_t r0 = 0; r0 < a.level; r0 += 2) {
+#pragma unroll 1
+    for (uint32_t P = 0; P < pairs; ++P) {
+      // first-pass slot q of thread tau is coefficient tau + q N/8 of owner q / 2
       uint32_t x[2][E];
 #pragma unroll
-      for (int pp = 0; pp < 2; ++pp)
-#pragma unroll
-        for (int q = 0; q < E; ++q) {
-          const uint32_t ad = dsmem_map(dig_s + ((r0 + pp) * Q + tau + (q % QE) * T) * 4u, q / QE);
-          x[pp][q] = static_cast<uint32_t>(dsmem_ld_s32(ad) + static_cast<int32_t>(p));  // (0, 2p)
+      for (int o = 0; o < 4; ++o) {
+        const uint32_t ad = dsmem_map(dig_t, o) + P * T * GRP_BYTES;
+        if constexpr (DIG16) {
+          const uint2 w = dsmem_ld_v2_u32(ad);
+          x[0][2 * o] = (w.x & 0xFFFFu) + dig_bias;
+          x[0][2 * o + 1] = (w.x >> 16) + dig_bias;
+          x[1][2 * o] = (w.y & 0xFFFFu) + dig_bias;
+          x[1][2 * o + 1] = (w.y >> 16) + dig_bias;
+        } else {
+          const uint4 w = dsmem_ld_v4_u32(ad);
+          x[0][2 * o] = w.x + dig_bias;
+          x[0][2 * o + 1] = w.y + dig_bias;
+          x[1][2 * o] = w.z + dig_bias;
+          x[1][2 * o + 1] = w.w + dig_bias;
         }
-      ntt_forward<LOGN, E, 2, 1>(x, tw, xb, tau, p);
-      const uint4 *g = reinterpret_cast<const uint4 *>(kbase + static_cast<size_t>(r0) * 2 * N + E * tau);
+      }
+      ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, p, CtaPairs());
+      const uint4 *g = reinterpret_cast<const uint4 *>(kbase + static_cast<size_t>(2 * P) * 2 * N + E * tau);
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t ga[E], gb[E];
@@ -167,97 +169,100 @@ __global__ void __launch_bounds__(TrShape<LOGN>::T) trace_kernel(const TraceArgs
         for (int e = 0; e < E; ++e) {
           const uint64_t prod = static_cast<uint64_t>(x[0][e]) * ga[e] + static_cast<uint64_t>(x[1][e]) * gb[e];
           const uint32_t rr = redc(prod, p, p_inv);
-          oh[c][e] = (r0 == 0) ? rr : cond_sub(oh[c][e] + rr, 4 * p);
+          oh[c][e] = (P == 0) ? rr : cond_sub(oh[c][e] + rr, 4 * p);
         }
       }
     }
-    ntt_inverse<LOGN, E, 2, 1>(oh, tw, xb, tau, p);
+    ntt_inverse<LOGN, E, 2, 2>(oh, tw, xb, tau, p, CtaPairs());
+    __syncthreads();  // every exchange read done: the buffer takes the outgoing residues
+    // (< 8p, CRT-scaled through the keys), one packed group (component, slot) per owner
 #pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-      for (int q = 0; q < E; ++q) {
-        const uint32_t y = oh[c][q];  // < 8p, CRT-scaled through the keys
-        dsmem_st_u32(dsmem_map(res_s + ((rank * 2 + c) * Q + tau + (q % QE) * T) * 4u, q / QE), y);
-      }
-    cluster.sync();
+    for (int o = 0; o < 4; ++o)
+      *reinterpret_cast<uint4 *>(xb + (o * T + tau) * 4) =
+          make_uint4(oh[0][2 * o], oh[0][2 * o + 1], oh[1][2 * o], oh[1][2 * o + 1]);
+    cluster_sync_shared();
 
-    // ---- phase 3: c <- c + (0 - X_0, sigma_k(B) - X_1) on the owned quarter ----
+    // ---- phase 3: c <- c + (0, sigma_k(B)) - X on the owned quarter ----
+    uint32_t yq[kPrimes][4];
 #pragma unroll
-    for (int m = 0; m < ITEMS; ++m) {
-      const uint32_t item = tau + m * T;
-      const uint32_t c = item / Q, jl = item % Q;
+    for (int pq = 0; pq < kPrimes; ++pq) {
+      const uint4 w = dsmem_ld_v4_u32(dsmem_map(res_t, pq));
+      yq[pq][0] = w.x;
+      yq[pq][1] = w.y;
+      yq[pq][2] = w.z;
+      yq[pq][3] = w.w;
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
       uint64_t sum = 0;
       uint32_t ysum = 0;
 #pragma unroll
       for (int pq = 0; pq < kPrimes; ++pq) {
-        const uint32_t y = res[(pq * 2 + c) * Q + jl];
+        const uint32_t y = yq[pq][m];
         sum += static_cast<uint64_t>(y) * a.cc.pr[pq].Mp_mod64;
         ysum += y >> 2;
       }
       const uint32_t u = crt_quotient(ysum);
-      const uint64_t X = sum - static_cast<uint64_t>(u) * a.cc.M_mod64;
-      if (PTMUL)
-        acc[c * Q + jl] = X + ((c == 1 && a.plain_add) ? a.plain_add[rank * Q + jl] : 0ull);
-      else
-        acc[c * Q + jl] += (c == 1 ? sig_b[jl] : 0ull) - X;
+      acc[(m / 2) * Q + tau + (m % 2) * T] -= sum - static_cast<uint64_t>(u) * a.cc.M_mod64;
     }
-    cluster.sync();
+    cluster_sync_shared();
   }
 
   uint64_t *gout = a.glwe_out + static_cast<size_t>(ct) * 2 * N;
 #pragma unroll
-  for (int m = 0; m < ITEMS; ++m) {
-    const uint32_t item = tau + m * T;
-    const uint32_t c = item / Q, jl = item % Q;
+  for (int m = 0; m < 4; ++m) {
+    const uint32_t c = m / 2, jl = tau + (m % 2) * T;
     gout[c * N + rank * Q + jl] = acc[c * Q + jl];
   }
   cluster.sync();
 }
 
-size_t trace_smem_bytes(uint32_t logN, uint32_t level) {
+static size_t trace_smem_bytes(uint32_t logN, uint32_t level, uint32_t base_log) {
   const size_t N = size_t(1) << logN, Q = N / 4;
-  size_t b = N * sizeof(uint2) + 3 * Q * sizeof(uint64_t) + kPrimes * 2 * Q * sizeof(uint32_t) +
-             (N + N / 8) * sizeof(uint32_t) + level * Q * sizeof(int32_t);
+  size_t b = N * sizeof(uint2) + 2 * Q * sizeof(uint64_t) + 2 * (N + N / 8) * sizeof(uint32_t) +
+             level * Q * (base_log <= 16 ? sizeof(uint16_t) : sizeof(uint32_t));
   return (b + 15) & ~size_t(15);
 }
 
-template <int LOGN, bool PTMUL>
+template <int LOGN, bool DIG16>
 static cudaError_t launch_trace_t(const TraceArgs &a, cudaStream_t s) {
-  auto kern = trace_kernel<LOGN, PTMUL>;
-  const size_t smem = trace_smem_bytes(LOGN, a.level);
+  auto kern = trace_kernel<LOGN, DIG16>;
+  const size_t smem = trace_smem_bytes(LOGN, a.level, a.base_log);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(4 * a.batch, 1, 1);
   cfg.blockDim = dim3(TrShape<LOGN>::T, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 4;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
+  attr[1].val.clusterSchedulingPolicyPreference = br_cluster_policy(kern, TrShape<LOGN>::T, smem, cfg.gridDim.x);
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-template <bool PTMUL>
-static cudaError_t launch_mode(const TraceArgs &a, uint32_t logN, cudaStream_t s) {
-  switch (logN) {
-    case 8: return launch_trace_t<8, PTMUL>(a, s);
-    case 9: return launch_trace_t<9, PTMUL>(a, s);
-    case 10: return launch_trace_t<10, PTMUL>(a, s);
-    case 11: return launch_trace_t<11, PTMUL>(a, s);
-    case 12: return launch_trace_t<12, PTMUL>(a, s);
-    default: return cudaErrorInvalidValue;
-  }
+template <int LOGN>
+static cudaError_t launch_trace_n(const TraceArgs &a, cudaStream_t s) {
+  return a.base_log <= 16 ? launch_trace_t<LOGN, true>(a, s) : launch_trace_t<LOGN, false>(a, s);
 }
 
-cudaError_t launch_trace(const TraceArgs &a, uint32_t logN, cudaStream_t s) { return launch_mode<false>(a, logN, s); }
-
-cudaError_t launch_plaintext_mul(const TraceArgs &a, uint32_t logN, cudaStream_t s) {
-  return launch_mode<true>(a, logN, s);
+cudaError_t launch_trace(const TraceArgs &a, uint32_t logN, cudaStream_t s) {
+  switch (logN) {
+    case 8: return launch_trace_n<8>(a, s);
+    case 9: return launch_trace_n<9>(a, s);
+    case 10: return launch_trace_n<10>(a, s);
+    case 11: return launch_trace_n<11>(a, s);
+    case 12: return launch_trace_n<12>(a, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // R <- (first ? 0 : R) + X^e r for `count` polynomials of N words (0 <= e < N):

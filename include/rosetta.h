@@ -315,7 +315,8 @@ int rosetta_selftest_wait_timeout(rosetta_ctx *ctx, uint32_t limit_us, void *str
 int rosetta_selftest_bounds(rosetta_ctx *ctx, void *stream);
 
 /* Wait for all work on `stream` and report any deferred execution error
- * (CUDA; TIMEOUT when a bounded wait of the tensor-core key switch gave up;
+ * (CUDA; TIMEOUT when a bounded wait of a tensor-core key switch or of the
+ * small-batch blind rotation gave up;
  * INVALID_ARG for an out-of-range LUT index seen by
  * rosetta_pbs_batch_multi_lut; BOUNDS when a check of a ROSETTA_DEBUG build
  * failed; the flag is cleared once reported).  Returns OK when the stream

@@ -87,4 +87,34 @@ __device__ __forceinline__ void dsmem_st_u32(uint32_t a, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
+// Asynchronous 16-byte store into another CTA's shared memory that adds its
+// bytes to the transaction count of an mbarrier there (both addresses mapped to
+// that CTA): whoever has waited for the mbarrier's phase sees the words.
+__device__ __forceinline__ void dsmem_st_async_v4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w,
+                                                  uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a),
+               "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+               : "memory");
+}
+
+// Wait for a phase of a local mbarrier that stores of the cluster's CTAs
+// complete; gives up after about two seconds.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, long long limit) {
+  uint32_t done;
+  const auto poll = [&] {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return done != 0u;
+  };
+  if (poll()) return true;
+  const long long t0 = clock64();
+  while (!poll())
+    if (clock64() - t0 > limit) return false;
+  return true;
+}
+
 }  // namespace rosetta

@@ -139,6 +139,10 @@ size_t br_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, bool dig16);
 bool br_solo_supported(uint32_t logN, uint32_t level, uint32_t base_log);
 size_t br_solo_smem_bytes(uint32_t n, uint32_t workers);
 cudaError_t launch_blind_rotate_solo(const BrArgs &a, uint32_t workers, cudaStream_t s);
+// small batches (blind_rotate_small.cu): two CTAs per prime, one per component
+bool br_small_supported(uint32_t logN, uint32_t level, uint32_t primes);
+size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes);
+cudaError_t launch_blind_rotate_small(const BrArgs &a, uint32_t logN, cudaStream_t s);
 // a.primes selects the kernel: the four-prime one or the three-prime one
 cudaError_t launch_blind_rotate(const BrArgs &a, uint32_t logN, bool dig16, cudaStream_t s);
 // three-prime kernel (blind_rotate3.cu): 16-bit digits, compiled ring sizes and levels only

@@ -99,6 +99,7 @@ extern "C" int rosetta_pbs_batch_noalloc(rosetta_ctx *c, const uint64_t *lwe_in,
   a.msg_bits = c->prm.msg_bits;
   a.batch = batch;
   a.num_luts = 1;
+  a.err_flag = c->d_err;
   cudaError_t e = run_blind_rotate(c, a, s);
   if (e != cudaSuccess) return ROSETTA_ERR_CUDA;
 

@@ -285,8 +285,21 @@ BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) 
 
 }  // namespace
 
-// Blind rotation of a batch: the cluster kernels, or at the standard ring, where
-// the context holds the float quotient's key, one worker per ciphertext for
+// Largest batch of the small-batch kernel: while its clusters find an SM for each
+// CTA (at N = 2048 15 clusters of 8 in GPCs of 18-20 SMs, at N = 4096 23 of 6), and
+// at the smaller rings while its CTAs of one or two warps do not crowd the SMs.
+// Measured against the cluster kernels: N = 2048, n = 742: 1 ciphertext 2.54 ms
+// against 3.78, 15: 2.57 / 3.50, 16: 4.14 / 3.50; N = 4096, n = 840: 1: 6.3 / 10.7,
+// 22: 6.0 / 9.8, 24: 12.0 / 9.8; N = 256, n = 64: 16: 145 us / 257, 128: 194 / 267,
+// 256: 359 / 333; N = 512, n = 64: 8: 283 / 578, 100: 550 / 750, 200: 1064 / 980.
+static uint32_t br_small_max(const rosetta_ctx *c) {
+  const uint32_t S = c->sms;
+  if (c->br_primes == kPrimes31) return c->logN == 12 ? S * 3 / 20 : 0;
+  return c->logN <= 9 ? S * 3 / 4 : c->logN == 10 ? S / 5 : S / 10;
+}
+
+// Blind rotation of a batch: the small-batch kernel, the cluster kernels, or at
+// the standard ring, where the context holds the float quotient's key, one worker per ciphertext for
 // whatever part of the batch fills the GPU.  A launch of w workers per SM takes
 // the same time for any number of ciphertexts up to w S (S SMs; measured at
 // n = 742: 9.7, 14.5, 20.6 ms for w = 1, 2, 3), the cluster kernel about in
@@ -295,7 +308,11 @@ BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) 
 // the rest r to as many workers as it needs, except where the cluster kernel
 // is still ahead: r <= 3/4 S and S < r <= 5/4 S.
 cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t s) {
-  if (!c->br_qf) return launch_blind_rotate(a, c->logN, c->dig16, s);
+  const auto cluster = [&](const BrArgs &b) {
+    return c->br_small && b.batch <= br_small_max(c) ? launch_blind_rotate_small(b, c->logN, s)
+                                                     : launch_blind_rotate(b, c->logN, c->dig16, s);
+  };
+  if (!c->br_qf) return cluster(a);
   const uint32_t S = c->sms, wave = 3 * S;
   uint32_t full = a.batch / wave * wave, rest = a.batch - full;
   if (rest > 2 * S) {
@@ -310,7 +327,7 @@ cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t
   cudaError_t e = full ? solo(0, full, 3) : cudaSuccess;
   if (e != cudaSuccess || rest == 0) return e;
   if (rest <= S - S / 4 || (rest > S && rest <= S + S / 4))
-    return launch_blind_rotate(br_slice(c, a, full, rest), c->logN, c->dig16, s);
+    return cluster(br_slice(c, a, full, rest));
   return solo(full, rest, rest <= S ? 1 : 2);
 }
 
@@ -379,6 +396,8 @@ int rosetta_params_init(rosetta_ctx **out, const rosetta_params *p, int cuda_dev
     const size_t smem3p = br3_smem_bytes(logN, p->pbs_level, p->lwe_dim, true);
     c->br3_pairs = smem3p <= (size_t)max_smem && per_sm(smem3p) >= per_sm(smem3);
   }
+  c->br_small = br_small_supported(logN, p->pbs_level, c->br_primes) &&
+                br_small_smem_bytes(logN, p->pbs_level, p->lwe_dim, c->br_primes) <= (size_t)max_smem;
   for (int q = 0; q < kPrimes; ++q)
     for (int m = 0; m < kTwLo; ++m) {
       c->tw_lo[q][m] = tw[((size_t)q << logN) + m];

@@ -283,6 +283,9 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
 #pragma unroll
     for (int e = 0; e < E; ++e)  // (28-bit primes: both below 4p)
       y[0][e] = P31 ? cond_sub(own[e], p) + cond_sub(got[e], p) : cond_sub(own[e] + got[e], 4 * p);
+    // the exchange buffer changes from pairs to single words, whose warp-local
+    // parts lie elsewhere: every forward read first
+    if constexpr (LEV != 1) __syncthreads();
     ntt_inverse<LOGN, E, 1, 1, P31>(y, tw, xb, tau, p, CtaThreads());  // CRT-scaled through the keys
 
     // ---- residues of the other primes, explicit CRT of component comp ----

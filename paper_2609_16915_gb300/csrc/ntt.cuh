@@ -412,7 +412,9 @@ __device__ __forceinline__ void xb_load(const uint32_t *buf, uint32_t (&v)[E], u
 }
 
 // The same for two polynomials whose words travel side by side (8-byte
-// elements, half the accesses): 2 pad elements after every 16 keep every pass
+// elements, half the accesses).  A warp's part of the buffer lies elsewhere than in
+// the single-word layout, so a kernel that changes layout between two exchanges
+// that synchronise warps only needs a barrier of its own there.  2 pad elements after every 16 keep every pass
 // free of bank conflicts (half-warps of 8-byte accesses, quarter-warps of the
 // last pass's 16-byte ones), and again the padding of base and offset adds.
 __host__ __device__ constexpr uint32_t xb_pad2(uint32_t i) { return i + ((i >> 4) << 1); }

@@ -9,14 +9,15 @@
 // > 2^111.99).  So a component takes two forward and one inverse transform per
 // prime, against the plaintext's two transformed rows.
 //
-// One CTA of N/8 threads per ciphertext, no cluster: thread tau owns
-// coefficients tau + e N/8, which are the transforms' first-pass slots, so words
-// are read and written once, straight between global memory and registers, and
-// nothing but the exchanges crosses threads.  The twiddles of one prime at a
-// time lie in shared memory.  128 registers: 16 warps per SM.  Measured, N =
-// 2048, 512 ciphertexts, the whole call with its host-side rows: 198 us with the
-// trace kernel's one-step mode (base 2^16 digits, eight rows whose cross-component
-// half was zero), 111 here.
+// One CTA of N/8 threads per ciphertext and component, no cluster: thread tau
+// owns coefficients tau + e N/8, which are the transforms' first-pass slots, so
+// words are read and written once, straight between global memory and registers,
+// and nothing but the exchanges crosses threads.  The twiddles of one prime at a
+// time lie in shared memory.  80 registers: 24 warps per SM at N = 2048.
+// Measured, N = 2048, 512 ciphertexts, the whole call with its host-side rows:
+// 198 us with the trace kernel's one-step mode (base 2^16 digits, eight rows whose
+// cross-component half was zero); 111 with one CTA of 128 registers for both
+// components (71 us of it the kernel: 1.7 waves of long CTAs); MEASURED here.
 #include <stdint.h>
 
 #include "internal.h"
@@ -25,7 +26,7 @@
 namespace rosetta {
 
 template <int LOGN>
-__global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 4096 >> LOGN)
+__global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >> LOGN))
     plain_mul_kernel(const __grid_constant__ PlainMulArgs a) {
   constexpr uint32_t N = 1u << LOGN, T = N / 8;
   constexpr int E = 8;
@@ -33,19 +34,17 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 4096 >> LOGN
   uint2 *tw_s = reinterpret_cast<uint2 *>(smem);
   uint32_t *xb = reinterpret_cast<uint32_t *>(tw_s + N);
   const uint32_t tau = threadIdx.x;
-  const uint64_t *gin = a.glwe_in + static_cast<size_t>(blockIdx.x) * 2 * N + tau;
+  const size_t poly = blockIdx.x;  // 2 ciphertext + component
+  const uint64_t *gin = a.glwe_in + poly * N + tau;
 
-  uint64_t w[2][E], s[2][E];
+  uint64_t w[E], s[E];
   uint32_t ysum[E];
 #pragma unroll
-  for (int c = 0; c < 2; ++c)
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      w[c][e] = gin[c * N + e * T] + ((1ull << 63) + (1ull << 31));  // both digits plus 2^31
-      s[c][e] = 0;
-    }
-#pragma unroll
-  for (int e = 0; e < E; ++e) ysum[e] = 0;
+  for (int e = 0; e < E; ++e) {
+    w[e] = gin[e * T] + ((1ull << 63) + (1ull << 31));  // both digits plus 2^31
+    s[e] = (poly & 1u) != 0 && a.plain_add ? a.plain_add[tau + e * T] : 0ull;
+    ysum[e] = 0;
+  }
 
 #pragma unroll 1
   for (uint32_t q = 0; q < kPrimes; ++q) {
@@ -57,50 +56,42 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 4096 >> LOGN
     for (uint32_t m = tau; m < N; m += T) tw_s[split_tw_slot<LOGN>(m)] = a.tw[q * N + m];
     __syncthreads();
     const SplitTw<LOGN, 3> tw{tw_s, a.tw_lo[q]};
-    uint32_t o[2][E];
+    uint32_t x[2][E];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      uint32_t x[2][E];
+    for (int e = 0; e < E; ++e) {
+      const uint32_t hi = static_cast<uint32_t>(w[e] >> 32), lo = static_cast<uint32_t>(w[e]);
+      x[0][e] = cond_sub(hi - (hi >> 28) * p, p) + bias;  // < 2p
+      x[1][e] = cond_sub(lo - (lo >> 28) * p, p) + bias;
+    }
+    ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, p, CtaPairs());
+    const uint4 *g = reinterpret_cast<const uint4 *>(a.keys + static_cast<size_t>(q) * 2 * N + E * tau);
+    uint32_t o[1][E];
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const uint32_t hi = static_cast<uint32_t>(w[c][e] >> 32), lo = static_cast<uint32_t>(w[c][e]);
-        x[0][e] = cond_sub(hi - (hi >> 28) * p, p) + bias;  // < 2p
-        x[1][e] = cond_sub(lo - (lo >> 28) * p, p) + bias;
-      }
-      ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, p, CtaPairs());
-      const uint4 *g = reinterpret_cast<const uint4 *>(a.keys + static_cast<size_t>(q) * 2 * N + E * tau);
+    for (int k = 0; k < E / 4; ++k) {
+      const uint4 v0 = __ldg(g + k), v1 = __ldg(g + N / 4 + k);
+      const uint32_t k0[4] = {v0.x, v0.y, v0.z, v0.w}, k1[4] = {v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-      for (int k = 0; k < E / 4; ++k) {
-        const uint4 v0 = __ldg(g + k), v1 = __ldg(g + N / 4 + k);
-        const uint32_t k0[4] = {v0.x, v0.y, v0.z, v0.w}, k1[4] = {v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const int e = 4 * k + m;
-          const uint64_t prod = static_cast<uint64_t>(cond_sub(x[0][e], 8 * p)) * k0[m] +
-                                static_cast<uint64_t>(cond_sub(x[1][e], 8 * p)) * k1[m];
-          o[c][e] = redc(prod, p, p_inv);
-        }
+      for (int m = 0; m < 4; ++m) {
+        const int e = 4 * k + m;
+        const uint64_t prod = static_cast<uint64_t>(cond_sub(x[0][e], 8 * p)) * k0[m] +
+                              static_cast<uint64_t>(cond_sub(x[1][e], 8 * p)) * k1[m];
+        o[0][e] = redc(prod, p, p_inv);
       }
     }
-    ntt_inverse<LOGN, E, 2, 2>(o, tw, xb, tau, p, CtaPairs());  // < 8p, CRT-scaled through the keys
+    // the exchange buffer changes from pairs to single words, whose warp-local
+    // parts lie elsewhere: every forward read first
+    __syncthreads();
+    ntt_inverse<LOGN, E, 1, 1>(o, tw, xb, tau, p, CtaThreads());  // < 8p, CRT-scaled through the keys
     const uint64_t mp = a.cc.pr[q].Mp_mod64;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      s[0][e] += static_cast<uint64_t>(o[0][e]) * mp;
-      s[1][e] += static_cast<uint64_t>(o[1][e]) * mp;
-      ysum[e] += qf_pack(o[0][e], o[1][e]);  // y >> 17 of both components; four add below 2^16
+      s[e] += static_cast<uint64_t>(o[0][e]) * mp;
+      ysum[e] += o[0][e] >> 2;
     }
   }
-  // quotient round(sum y / p): y / 2^28 undershoots by less than 2^-5 in all, the
-  // dropped bits by 2^-9, and |X| / M < 2^-4
-  uint64_t *gout = a.glwe_out + static_cast<size_t>(blockIdx.x) * 2 * N + tau;
+  uint64_t *gout = a.glwe_out + poly * N + tau;
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const uint32_t u0 = ((ysum[e] & 0xFFFFu) + (1u << 10)) >> 11, u1 = ((ysum[e] >> 16) + (1u << 10)) >> 11;
-    gout[e * T] = s[0][e] - static_cast<uint64_t>(u0) * a.cc.M_mod64;
-    gout[N + e * T] =
-        s[1][e] - static_cast<uint64_t>(u1) * a.cc.M_mod64 + (a.plain_add ? a.plain_add[tau + e * T] : 0ull);
-  }
+  for (int e = 0; e < E; ++e) gout[e * T] = s[e] - static_cast<uint64_t>(crt_quotient(ysum[e])) * a.cc.M_mod64;
 }
 
 template <int LOGN>
@@ -112,7 +103,7 @@ static cudaError_t launch_pm_t(const PlainMulArgs &a, uint32_t batch, cudaStream
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  kern<<<batch, N / 8, smem, s>>>(a);
+  kern<<<2 * batch, N / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
   uint16_t *atil = reinterpret_cast<uint16_t *>(dig + 2 * level * Q);  // [n+1]
 
   const uint32_t p = a.cc.pr[rank].p;
+  const NttPrime np(a.cc.pr[rank]);
   const uint32_t p_inv = a.cc.pr[rank].p_inv;
 
   // ---- set-up: twiddles, modulus switch, accumulator ----
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
           for (int h = 0; h < QE; ++h)
             x[pp][o * QE + h] = static_cast<uint32_t>(d[pp * QE + h] + static_cast<int32_t>(p));  // in (0, 2p)
       }
-      ntt_forward<LOGN, E, 2, XBUF>(x, tw, xb, tau, p, TH());
+      ntt_forward<LOGN, E, 2, XBUF>(x, tw, xb, tau, np, TH());
       // BSK_i words of this prime for rows r0, r0+1, E per thread and
       // component, contiguous across the CTA (16-byte loads)
       const uint4 *g = reinterpret_cast<const uint4 *>(gbase + static_cast<size_t>(r0) * 2 * N + E * tau);
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
 #pragma unroll
           for (int pp = 0; pp < 2; ++pp)
 #pragma unroll
-            for (int e = 0; e < E; ++e) x[pp][e] = cond_sub(x[pp][e], 8 * p);  // < 16p -> < 8p
+            for (int e = 0; e < E; ++e) x[pp][e] = cond_sub(x[pp][e], np.p8);  // < 16p -> < 8p
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
         }
       }
     }
-    ntt_inverse<LOGN, E, 2, XBUF>(oh, tw, xb, tau, p, TH());
+    ntt_inverse<LOGN, E, 2, XBUF>(oh, tw, xb, tau, np, TH());
     __syncthreads();  // every exchange read done: the buffer takes the outgoing residues
     // CRT-scaled residues (< 8p; the keys carry the CRT factor), one packed
     // group (component, h) per owner

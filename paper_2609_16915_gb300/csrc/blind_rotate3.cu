@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
   uint16_t *atil = reinterpret_cast<uint16_t *>(dig4 + L * T);
 
   const uint32_t p = a.cc.pr[rank].p;
+  const NttPrime np(a.cc.pr[rank]);
   const uint32_t p_inv = a.cc.pr[rank].p_inv;
   const uint32_t s0 = 3 * rank;   // first owned slot
   const bool three = rank < 2;    // owners 0 and 1 hold a third slot
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
           x[1][q + 2] = hi16(w4) + dig_bias;
         }
       }
-      ntt_forward<LOGN, E, 2, XBUF, true>(x, tw, xb, tau, p, TH());  // outputs in [0, 2p)
+      ntt_forward<LOGN, E, 2, XBUF, true>(x, tw, xb, tau, np, TH());  // outputs in [0, 2p)
       // below p, so that a row pair's two products sum below 2 p^2 < p 2^32
 #pragma unroll
       for (int pp = 0; pp < 2; ++pp)
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(Br3Shape<LOGN>::T, Br3Shape<LOGN>::MIN_CTAS) b
         }
       }
     }
-    ntt_inverse<LOGN, E, 2, XBUF, true>(oh, tw, xb, tau, p, TH());  // outputs in [0, 2p)
+    ntt_inverse<LOGN, E, 2, XBUF, true>(oh, tw, xb, tau, np, TH());  // outputs in [0, 2p)
     // CRT-scaled residues (the keys carry the CRT factor): one packed group
     // per other owner, left in this CTA's exchange buffer (once every thread
     // has finished the transforms' last exchange) at the owner's index among

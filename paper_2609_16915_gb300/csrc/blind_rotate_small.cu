@@ -22,7 +22,8 @@
 // Measured, n = 742, N = 2048, one ciphertext: 3.78 ms with four CTAs and three
 // cluster barriers per step (blind_rotate.cu); 3.92 with the whole accumulator in
 // every one of four CTAs and one barrier (the arithmetic, not the barriers, is
-// most of a step); 2.85 with two CTAs per prime and two barriers; 2.54 here.
+// most of a step); 2.85 with two CTAs per prime and two barriers; 2.54 with
+// st.async, 2.42 with 2p and 8p loaded as values (NttPrime).
 //
 // Every wait gives up after about two seconds and raises the error flag; the CTA
 // then runs on without waiting.
@@ -128,6 +129,7 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
   uint16_t *atil = reinterpret_cast<uint16_t *>(res + 2 * (PRIMES - 1) * 2 * T);
 
   const uint32_t p = a.cc.pr[q].p;
+  const NttPrime npr(a.cc.pr[q]);
   const uint32_t p_inv = a.cc.pr[q].p_inv;
   const uint32_t level = LEV > 0 ? static_cast<uint32_t>(LEV) : a.level;
 
@@ -237,11 +239,11 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
 #pragma unroll
         for (int e = 0; e < E; ++e)
           x[r][e] = lev + r < level ? biased_digit(w[e], a.base_log, lev + r) + dig_bias : p;
-      ntt_forward<LOGN, E, NP, NP, P31>(x, tw, xb, tau, p, TH());
+      ntt_forward<LOGN, E, NP, NP, P31>(x, tw, xb, tau, npr, TH());
 #pragma unroll
       for (int r = 0; r < NP; ++r)
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[r][e] = cond_sub(x[r][e], P31 ? p : 8 * p);
+        for (int e = 0; e < E; ++e) x[r][e] = cond_sub(x[r][e], P31 ? p : npr.p8);
       mac<P31, NP>(oth, x, k, 1, first, p, p_inv);
       between();
       mac<P31, NP>(own, x, k, 0, first, p, p_inv);
@@ -286,7 +288,7 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
     // the exchange buffer changes from pairs to single words, whose warp-local
     // parts lie elsewhere: every forward read first
     if constexpr (LEV != 1) __syncthreads();
-    ntt_inverse<LOGN, E, 1, 1, P31>(y, tw, xb, tau, p, CtaThreads());  // CRT-scaled through the keys
+    ntt_inverse<LOGN, E, 1, 1, P31>(y, tw, xb, tau, npr, CtaThreads());  // CRT-scaled through the keys
 
     // ---- residues of the other primes, explicit CRT of component comp ----
 #pragma unroll

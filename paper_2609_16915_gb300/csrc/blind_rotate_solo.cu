@@ -23,14 +23,15 @@
 // last, when the digits' registers are free.
 //
 // What bounds it: at three workers (24 warps, 80 registers, no spills) the
-// shared-memory pipe is 68 %, the integer-multiply pipe 67 % and the issue
-// slots 64 % busy.  Hence the layouts: both polynomials of a transform cross the
+// shared-memory pipe, the integer-multiply pipe and the issue slots are each about
+// two thirds busy.  Hence the layouts: both polynomials of a transform cross the
 // exchange buffer as 8-byte pairs, all four float planes as 16-byte elements,
 // both components of an accumulator word lie together, and the first six
 // stages' twiddles come from the constant bank.  Measured, n = 742, batch 4096:
 // 235.9 ms with the cluster kernel; here 219.3 with the float transforms
-// first and spills (172 bytes), 190.1 without, 184.5 with the paired exchanges
-// (456 ciphertexts, one wave: 28.8, 24.5, 21.2, 20.6 ms).  Two workers with 128
+// first and spills (172 bytes), 190.1 without, 184.5 with the paired exchanges,
+// 171 with 2p and 8p loaded as values (NttPrime: 6079 -> 5470 instructions a step;
+// 456 ciphertexts, one wave: 28.8, 24.5, 21.2, 20.6, 19.1 ms).  Two workers with 128
 // registers: 14.9 ms per 304.  The float quotient as the fourth CTA of a
 // cluster gained 1.6 % only: a cluster moves at the pace of its most loaded SM.
 #include <stdint.h>
@@ -176,18 +177,19 @@ __global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(cons
         q = q == kPrimesQf - 1 ? 0 : q + 1;
       }
       const uint32_t p = a.cc.pr[q].p, p_inv = a.cc.pr[q].p_inv;
+      const NttPrime np(a.cc.pr[q]);
       const SplitTw<kLogN, 6> tw{tw_all + q * N, a.tw_lo[q]};
       uint32_t x[2][E];
 #pragma unroll
       for (int pp = 0; pp < 2; ++pp)
 #pragma unroll
         for (int e = 0; e < E; ++e) x[pp][e] = static_cast<uint32_t>(d[pp][e]) + p;  // in (0, 2p)
-      ntt_forward<kLogN, E, 2, 2>(x, tw, xb, tau, p, th);
+      ntt_forward<kLogN, E, 2, 2>(x, tw, xb, tau, np, th);
       const uint4 *g = reinterpret_cast<const uint4 *>(key + q * kblk + E * tau);
 #pragma unroll
       for (int pp = 0; pp < 2; ++pp)
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[pp][e] = cond_sub(x[pp][e], 8 * p);  // < 16p -> < 8p
+        for (int e = 0; e < E; ++e) x[pp][e] = cond_sub(x[pp][e], np.p8);  // < 16p -> < 8p
 #pragma unroll
       for (int h = 0; h < E / 4; ++h) {
         uint4 w[2][2];  // [component][row]
@@ -210,7 +212,7 @@ __global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(cons
           }
         }
       }
-      ntt_inverse<kLogN, E, 2, 2>(y, tw, xb, tau, p, th);  // < 8p, CRT-scaled through the keys
+      ntt_inverse<kLogN, E, 2, 2>(y, tw, xb, tau, np, th);  // < 8p, CRT-scaled through the keys
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const uint32_t t = qf_pack(y[0][e], y[1][e]);

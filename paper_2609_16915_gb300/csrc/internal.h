@@ -31,7 +31,7 @@ constexpr int kQfShift = 16;
 constexpr int kQfBits = 98;
 
 struct PrimeConsts {
-  uint32_t p;
+  uint32_t p, p2, p8;  // the prime; 2p and 8p (28-bit set; modulo 2^32 otherwise)
   uint32_t p_inv;     // p^{-1} mod 2^32 (Montgomery reduction)
   uint32_t crt_c;     // N^{-1} * (M/p)^{-1} mod p (folded into the transformed keys)
   uint32_t crt_cs;    // Shoup companion of crt_c

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
 #pragma unroll 1
   for (uint32_t q = 0; q < kPrimes; ++q) {
     const uint32_t p = a.cc.pr[q].p, p_inv = a.cc.pr[q].p_inv;
+  const NttPrime np(a.cc.pr[q]);
     // digit u - 2^31 mod p: u = (u >> 28) 2^28 + .., 2^28 = p + g with g < 2^18;
     // 2^31 = 8p + 8g
     const uint32_t bias = p - 8 * ((1u << 28) - p);
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
       x[0][e] = cond_sub(hi - (hi >> 28) * p, p) + bias;  // < 2p
       x[1][e] = cond_sub(lo - (lo >> 28) * p, p) + bias;
     }
-    ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, p, CtaPairs());
+    ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, np, CtaPairs());
     const uint4 *g = reinterpret_cast<const uint4 *>(a.keys + static_cast<size_t>(q) * 2 * N + E * tau);
     uint32_t o[1][E];
 #pragma unroll
@@ -73,15 +74,15 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         const int e = 4 * k + m;
-        const uint64_t prod = static_cast<uint64_t>(cond_sub(x[0][e], 8 * p)) * k0[m] +
-                              static_cast<uint64_t>(cond_sub(x[1][e], 8 * p)) * k1[m];
+        const uint64_t prod = static_cast<uint64_t>(cond_sub(x[0][e], np.p8)) * k0[m] +
+                              static_cast<uint64_t>(cond_sub(x[1][e], np.p8)) * k1[m];
         o[0][e] = redc(prod, p, p_inv);
       }
     }
     // the exchange buffer changes from pairs to single words, whose warp-local
     // parts lie elsewhere: every forward read first
     __syncthreads();
-    ntt_inverse<LOGN, E, 1, 1>(o, tw, xb, tau, p, CtaThreads());  // < 8p, CRT-scaled through the keys
+    ntt_inverse<LOGN, E, 1, 1>(o, tw, xb, tau, np, CtaThreads());  // < 8p, CRT-scaled through the keys
     const uint64_t mp = a.cc.pr[q].Mp_mod64;
 #pragma unroll
     for (int e = 0; e < E; ++e) {

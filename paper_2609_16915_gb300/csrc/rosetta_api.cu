@@ -288,8 +288,8 @@ BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) 
 // Largest batch of the small-batch kernel: while its clusters find an SM for each
 // CTA (at N = 2048 15 clusters of 8 in GPCs of 18-20 SMs, at N = 4096 23 of 6), and
 // at the smaller rings while its CTAs of one or two warps do not crowd the SMs.
-// Measured against the cluster kernels: N = 2048, n = 742: 1 ciphertext 2.54 ms
-// against 3.78, 15: 2.57 / 3.50, 16: 4.14 / 3.50; N = 4096, n = 840: 1: 6.3 / 10.7,
+// Measured against the cluster kernels as they were then: N = 2048, n = 742: 1
+// ciphertext 2.54 ms against 3.78, 15: 2.57 / 3.50, 16: 4.14 / 3.50; N = 4096, n = 840: 1: 6.3 / 10.7,
 // 22: 6.0 / 9.8, 24: 12.0 / 9.8; N = 256, n = 64: 16: 145 us / 257, 128: 194 / 267,
 // 256: 359 / 333; N = 512, n = 64: 8: 283 / 578, 100: 550 / 750, 200: 1064 / 980.
 static uint32_t br_small_max(const rosetta_ctx *c) {
@@ -302,9 +302,9 @@ static uint32_t br_small_max(const rosetta_ctx *c) {
 // the standard ring, where the context holds the float quotient's key, one worker per ciphertext for
 // whatever part of the batch fills the GPU.  A launch of w workers per SM takes
 // the same time for any number of ciphertexts up to w S (S SMs; measured at
-// n = 742: 9.7, 14.5, 20.6 ms for w = 1, 2, 3), the cluster kernel about in
-// proportion to its number (95: 7.8, 114: 9.7, 152: 10.9, 190: 14.4, 228: 15.8,
-// 304: 19.9 ms; at 456 28.8).  So whole waves of 3 S go to three workers, and
+// n = 742, with the key switch: 8.6, 13.4, 19.1 ms for w = 1, 2, 3), the cluster
+// kernel about in proportion to its number (95: 6.5, 114: 8.1, 153: 10.2, 190:
+// 11.9 ms).  So whole waves of 3 S go to three workers, and
 // the rest r to as many workers as it needs, except where the cluster kernel
 // is still ahead: r <= 3/4 S and S < r <= 5/4 S.
 cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t s) {

@@ -94,6 +94,8 @@ bool build_tables(uint32_t logN, uint32_t primes, uint2 *tw_host, CrtConsts *cc,
     }
     PrimeConsts &pc = cc->pr[q];
     pc.p = p;
+    pc.p2 = 2 * p;
+    pc.p8 = 8 * p;
     uint32_t inv = 1;  // Newton iteration for p^{-1} mod 2^32
     for (int it = 0; it < 5; ++it) inv *= 2u - p * inv;
     pc.p_inv = inv;

@@ -26,7 +26,7 @@
 // memory only, as in the blind rotation; the transforms exchange pairs; four
 // CTAs fit an SM at N = 2048.  Measured, N = 2048, gadget 2^16 x 4, 1024
 // ciphertexts: 1.84 ms with single-word exchanges, pushed residues and plain
-// barriers, 1.38 ms here.
+// barriers, 1.38 ms with these, 1.25 with 2p and 8p loaded as values (NttPrime).
 #include <cooperative_groups.h>
 
 #include "dsmem.cuh"
@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(TrShape<LOGN>::T, TrShape<LOGN>::MIN_CTAS) tra
   uint32_t *dig = xb + B::XB_WORDS;                           // [level / 2][T][2 rows][2 slots], 16- or 32-bit
 
   const uint32_t p = a.cc.pr[rank].p;
+  const NttPrime np(a.cc.pr[rank]);
   const uint32_t p_inv = a.cc.pr[rank].p_inv;
 
   for (uint32_t m = tau; m < N; m += T) tw_s[split_tw_slot<LOGN>(m)] = a.tw[rank * N + m];
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(TrShape<LOGN>::T, TrShape<LOGN>::MIN_CTAS) tra
           x[1][2 * o + 1] = w.w + dig_bias;
         }
       }
-      ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, p, CtaPairs());
+      ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, np, CtaPairs());
       const uint4 *g = reinterpret_cast<const uint4 *>(kbase + static_cast<size_t>(2 * P) * 2 * N + E * tau);
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(TrShape<LOGN>::T, TrShape<LOGN>::MIN_CTAS) tra
 #pragma unroll
           for (int pp = 0; pp < 2; ++pp)
 #pragma unroll
-            for (int e = 0; e < E; ++e) x[pp][e] = cond_sub(x[pp][e], 8 * p);
+            for (int e = 0; e < E; ++e) x[pp][e] = cond_sub(x[pp][e], np.p8);
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(TrShape<LOGN>::T, TrShape<LOGN>::MIN_CTAS) tra
         }
       }
     }
-    ntt_inverse<LOGN, E, 2, 2>(oh, tw, xb, tau, p, CtaPairs());
+    ntt_inverse<LOGN, E, 2, 2>(oh, tw, xb, tau, np, CtaPairs());
     __syncthreads();  // every exchange read done: the buffer takes the outgoing residues
     // (< 8p, CRT-scaled through the keys), one packed group (component, slot) per owner
 #pragma unroll

@@ -136,6 +136,15 @@ def br_launches(p, batch, sms) -> int:
     return 2
 
 
+def lookup_launches(p, batch, n_seg, sms) -> int:
+    """Kernels of one segmented lookup: the segments go in groups of up to 4096
+    ciphertexts (product, rotation, trace, accumulation each), with one product
+    and rotation before and one product, rotation and trace after."""
+    group = min(n_seg, max(1, 4096 // batch))
+    sizes = [min(group, n_seg - s) for s in range(0, n_seg, group)]
+    return 5 + 2 * br_launches(p, batch, sms) + sum(3 + br_launches(p, m * batch, sms) for m in sizes)
+
+
 def ks_fp8(p) -> bool:
     """Does the library take the 8-bit tensor-core key switch (every batch)?"""
     return p.ks_base_log <= 5 and p.kN % 128 == 0 and 2 ** (p.ks_base_log - 1) * 16 * p.kN * p.ks_level < 2 ** 24
@@ -400,7 +409,7 @@ def run_lookup(args, p, batch, torch, dev, R, clock_sampler):
                      "kernel_ms": br_ms, "trace_ms": tr_ms,
                      "path_ops_per_lookup": ops, "path_achieved": path_achieved,
                      "path_frac": path_achieved / alu_peak},
-        "gpu_launches": ((n_seg + 2) * (1 + br_launches(p, batch, sms)) + (n_seg + 1) + n_seg + 2) * args.steps,
+        "gpu_launches": lookup_launches(p, batch, n_seg, sms) * args.steps,
         "clocks": clk.summary(),
     }
     return line

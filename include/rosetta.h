@@ -266,7 +266,9 @@ int rosetta_upload_lookup_table(rosetta_ctx *ctx, uint32_t n_seg, const int64_t 
  *           others ~ 0 (each Trace multiplies by N: N has no inverse mod 2^64)
  * Needs the BSK, KSK, trace keys and lookup tables.  Stream-ordered, no host
  * synchronisation.  Per ciphertext: n_seg + 2 plaintext products, n_seg + 2
- * blind rotations, one key switch, n_seg + 1 traces.  Errors: INVALID_ARG,
+ * blind rotations, one key switch, n_seg + 1 traces; the segments' products,
+ * rotations and traces share launches, up to 4096 ciphertexts each, with
+ * scratch for as many (2 x 2N words each).  Errors: INVALID_ARG,
  * KEYS_MISSING, CUDA, OOM. */
 int rosetta_segmented_lookup_batch(rosetta_ctx *ctx, const uint64_t *glwe_x, const uint64_t *lwe_seg, uint32_t batch,
                                    uint64_t *glwe_out, void *stream);

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(BrShape<LOGN>::T, BrShape<LOGN>::MIN_CTAS) bli
   // ---- set-up: twiddles, modulus switch, accumulator ----
   for (uint32_t m = tau; m < N; m += T) tw_s[tw_slot<LOGN, PAIRS>(m)] = a.tw[rank * N + m];
   const auto tw = make_tw<LOGN, PAIRS>(tw_s, a.tw_lo[rank]);
-  const uint64_t *lwe = a.lwe_in + static_cast<size_t>(ct) * (a.n + 1);
+  const uint64_t *lwe = a.lwe_in + static_cast<size_t>((a.lwe_first + ct) % a.lwe_count) * (a.n + 1);
   constexpr uint32_t SH = 63 - LOGN;  // 64 - log2(2N)
   for (uint32_t i = tau; i <= a.n; i += T)
     atil[i] = static_cast<uint16_t>(((lwe[i] + (1ull << (SH - 1))) >> SH) & (TWO_N - 1));

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kWorkers *kT, 1) blind_rotate_solo_kernel(cons
   if (ct >= a.batch) return;  // the whole worker; from here on it meets only its own barrier
   const GroupThreads th{worker + 1u, T};
 
-  const uint64_t *lwe = a.lwe_in + static_cast<size_t>(ct) * (a.n + 1);
+  const uint64_t *lwe = a.lwe_in + static_cast<size_t>((a.lwe_first + ct) % a.lwe_count) * (a.n + 1);
   constexpr uint32_t SH = 63 - kLogN;  // 64 - log2(2N)
   for (uint32_t i = tau; i <= a.n; i += T)
     atil[i] = static_cast<uint16_t>(((lwe[i] + (1ull << (SH - 1))) >> SH) & (TWO_N - 1));

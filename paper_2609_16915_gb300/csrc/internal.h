@@ -49,7 +49,10 @@ struct CrtConsts {
 constexpr int kTwLo = 64;  // entries of the first six stages
 
 struct BrArgs {
-  const uint64_t *lwe_in;   // [batch][n+1]
+  // ciphertext ct takes LWE (lwe_first + ct) mod lwe_count: several test
+  // polynomials may share one rotation index
+  const uint64_t *lwe_in;   // [lwe_count][n+1]
+  uint32_t lwe_count, lwe_first;
   const uint64_t *lut;      // [num_luts][2^p]; ignored when glwe_in is set
   uint64_t *lwe_big_out;    // [batch][N+1] extracted LWEs (k = 1), or
   uint64_t *glwe_out;       // [batch][2][N] rotated accumulators (when set)
@@ -94,12 +97,14 @@ struct TraceArgs {
   CrtConsts cc;
 };
 
-// (P A, P B + Q): P by the transformed rows of P 2^32 and P.
+// (P_i A, P_i B + Q_i) for `polys` plaintexts: P by the transformed rows of P 2^32
+// and P.
 struct PlainMulArgs {
   const uint64_t *glwe_in;    // [batch][2][N]
-  uint64_t *glwe_out;         // [batch][2][N]
-  const uint32_t *keys;       // transform domain [prime][2][N]
-  const uint64_t *plain_add;  // Q [N], or null
+  uint64_t *glwe_out;         // [polys][batch][2][N]
+  const uint32_t *keys;       // transform domain [polys][prime][2][N]
+  const uint64_t *plain_add;  // Q [polys][N], or null
+  uint32_t batch, polys;
   const uint2 *tw;            // [prime][N]
   uint2 tw_lo[kPrimes][8];
   CrtConsts cc;
@@ -162,9 +167,10 @@ cudaError_t launch_key_transform(const uint64_t *raw, uint32_t *out, const uint2
                                  uint32_t logN, uint32_t count, uint32_t rows, cudaStream_t s,
                                  uint32_t primes = kPrimes);
 cudaError_t launch_trace(const TraceArgs &a, uint32_t logN, cudaStream_t s);
-cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, uint32_t batch, cudaStream_t s);
-cudaError_t launch_monomial_acc(uint64_t *R, const uint64_t *r, uint32_t count, uint32_t logN, uint32_t e, bool first,
-                                cudaStream_t s);
+cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, cudaStream_t s);
+// R (+)= sum_i X^(e0 + i step) r_i for i < polys: r [polys][count][N], R [count][N]
+cudaError_t launch_monomial_acc(uint64_t *R, const uint64_t *r, uint32_t count, uint32_t logN, uint32_t polys, uint32_t e0,
+                                uint32_t step, bool first, cudaStream_t s);
 uint32_t ks_tc_limbs(uint32_t kN, uint32_t level, uint32_t base_log);  // 8, 16, or 0 (not exact)
 size_t ks_tc_b_words16(uint32_t kN, uint32_t level, uint32_t n, uint32_t limbs);
 size_t ks_tc_a_words16(uint32_t batch, uint32_t kN, uint32_t level);

@@ -90,6 +90,7 @@ extern "C" int rosetta_pbs_batch_noalloc(rosetta_ctx *c, const uint64_t *lwe_in,
 
   BrArgs a{};
   a.lwe_in = lwe_in;
+  a.lwe_count = batch;
   a.lut = lut;
   a.lwe_big_out = big;
   br_key_args(c, &a);

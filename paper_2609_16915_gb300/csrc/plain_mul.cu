@@ -9,7 +9,7 @@
 // > 2^111.99).  So a component takes two forward and one inverse transform per
 // prime, against the plaintext's two transformed rows.
 //
-// One CTA of N/8 threads per ciphertext and component, no cluster: thread tau
+// One CTA of N/8 threads per plaintext, ciphertext and component, no cluster: thread tau
 // owns coefficients tau + e N/8, which are the transforms' first-pass slots, so
 // words are read and written once, straight between global memory and registers,
 // and nothing but the exchanges crosses threads.  The twiddles of one prime at a
@@ -34,15 +34,17 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
   uint2 *tw_s = reinterpret_cast<uint2 *>(smem);
   uint32_t *xb = reinterpret_cast<uint32_t *>(tw_s + N);
   const uint32_t tau = threadIdx.x;
-  const size_t poly = blockIdx.x;  // 2 ciphertext + component
+  const uint32_t which = blockIdx.x / (2 * a.batch);           // plaintext
+  const size_t poly = blockIdx.x - which * (2 * a.batch);      // 2 ciphertext + component
   const uint64_t *gin = a.glwe_in + poly * N + tau;
+  const uint64_t *add = (poly & 1u) != 0 && a.plain_add ? a.plain_add + static_cast<size_t>(which) * N : nullptr;
 
   uint64_t w[E], s[E];
   uint32_t ysum[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     w[e] = gin[e * T] + ((1ull << 63) + (1ull << 31));  // both digits plus 2^31
-    s[e] = (poly & 1u) != 0 && a.plain_add ? a.plain_add[tau + e * T] : 0ull;
+    s[e] = add ? add[tau + e * T] : 0ull;
     ysum[e] = 0;
   }
 
@@ -65,7 +67,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
       x[1][e] = cond_sub(lo - (lo >> 28) * p, p) + bias;
     }
     ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, np, CtaPairs());
-    const uint4 *g = reinterpret_cast<const uint4 *>(a.keys + static_cast<size_t>(q) * 2 * N + E * tau);
+    const uint4 *g = reinterpret_cast<const uint4 *>(a.keys + (static_cast<size_t>(which) * kPrimes + q) * 2 * N + E * tau);
     uint32_t o[1][E];
 #pragma unroll
     for (int k = 0; k < E / 4; ++k) {
@@ -90,13 +92,13 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
       ysum[e] += o[0][e] >> 2;
     }
   }
-  uint64_t *gout = a.glwe_out + poly * N + tau;
+  uint64_t *gout = a.glwe_out + static_cast<size_t>(blockIdx.x) * N + tau;
 #pragma unroll
   for (int e = 0; e < E; ++e) gout[e * T] = s[e] - static_cast<uint64_t>(crt_quotient(ysum[e])) * a.cc.M_mod64;
 }
 
 template <int LOGN>
-static cudaError_t launch_pm_t(const PlainMulArgs &a, uint32_t batch, cudaStream_t s) {
+static cudaError_t launch_pm_t(const PlainMulArgs &a, cudaStream_t s) {
   constexpr size_t N = size_t(1) << LOGN;
   const size_t smem = N * sizeof(uint2) + 2 * (N + N / 8) * sizeof(uint32_t);
   auto kern = plain_mul_kernel<LOGN>;
@@ -104,17 +106,17 @@ static cudaError_t launch_pm_t(const PlainMulArgs &a, uint32_t batch, cudaStream
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  kern<<<2 * batch, N / 8, smem, s>>>(a);
+  kern<<<2 * a.batch * a.polys, N / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, uint32_t batch, cudaStream_t s) {
+cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, cudaStream_t s) {
   switch (logN) {
-    case 8: return launch_pm_t<8>(a, batch, s);
-    case 9: return launch_pm_t<9>(a, batch, s);
-    case 10: return launch_pm_t<10>(a, batch, s);
-    case 11: return launch_pm_t<11>(a, batch, s);
-    case 12: return launch_pm_t<12>(a, batch, s);
+    case 8: return launch_pm_t<8>(a, s);
+    case 9: return launch_pm_t<9>(a, s);
+    case 10: return launch_pm_t<10>(a, s);
+    case 11: return launch_pm_t<11>(a, s);
+    case 12: return launch_pm_t<12>(a, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -369,6 +369,208 @@ size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t p
   return brs_smem(size_t(1) << logN, level == 1 && logN >= 11, n, primes);
 }
 
+// ---------------------------------------------------------------------------- the smallest ring
+//
+// N = 256 beyond a few dozen ciphertexts: the whole cluster's work in one CTA per
+// ciphertext, a warp per prime and component, so that what the cluster sends through
+// distributed shared memory goes through the CTA's own, and an SM holds two
+// ciphertexts (16 warps) instead of clusters of one-warp CTAs that wait for each
+// other.  The accumulator is there once; each warp does the CRT of a quarter of its
+// component.  Three CTA barriers per step.  Bounded by the latency of a step (2.5 us)
+// up to two ciphertexts per SM, by the integer multiplies and the barriers beyond.
+// Measured with the key switch, n = 64, level 2, against the four-CTA cluster kernel:
+// 152 ciphertexts 172 us (312), 304: 273 (527), 2000: 1.61 ms (1.97), 20000: 14.8 (18.4).
+// Three CTAs per SM (85 registers): 1.64 / 14.98 ms; four (64, spilling): 1.68 / 15.15.  The
+// same at N = 512 (two warps per group, six levels, n = 64): 600 us against 515 at 100
+// ciphertexts, 7.98 ms against 7.14 at 2000: not built there.
+struct BrtShape {
+  static constexpr int LOGN = 8, N = 1 << LOGN, T = N / 8, GROUPS = 2 * kPrimes, THREADS = GROUPS * T;
+  static constexpr int XB_WORDS = 2 * (N + N / 8);  // per group
+};
+
+// Shared memory: twiddles uint2 [4][N], acc uint64 [2][N], exchange buffers
+// [8][2 (N + N/8)], partial products uint32 [8][N], residues uint32 [4][2][N],
+// switched mask and body uint16 [n+1].
+size_t br_tiny_smem_bytes(uint32_t n) {
+  constexpr size_t N = BrtShape::N;
+  return (kPrimes * N * sizeof(uint2) + 2 * N * sizeof(uint64_t) + 8 * 2 * (N + N / 8) * sizeof(uint32_t) +
+          8 * N * sizeof(uint32_t) + 8 * N * sizeof(uint32_t) + (n + 1) * sizeof(uint16_t) + 15) & ~size_t(15);
+}
+
+template <int LEV>
+__global__ void __launch_bounds__(BrtShape::THREADS, 2)
+    blind_rotate_tiny_kernel(const __grid_constant__ BrArgs a) {
+  using B = BrtShape;
+  constexpr uint32_t LOGN = B::LOGN, N = B::N, T = B::T, TWO_N = 2 * N;
+  constexpr int E = 8;
+  const uint32_t group = __shfl_sync(0xffffffffu, threadIdx.x / T, 0);  // (warp-uniform for the compiler)
+  const uint32_t tau = threadIdx.x % T, q = group / 2, comp = group % 2;
+  const uint32_t ct = blockIdx.x;
+  if (!dbg_ok(ct < a.batch, a.err_flag)) return;
+  const GroupThreads pairs{group + 1u, T};
+  const GroupSingles singles{group + 1u, T};
+
+  extern __shared__ __align__(16) unsigned char smem[];
+  uint2 *tw_s = reinterpret_cast<uint2 *>(smem);
+  uint64_t *acc_all = reinterpret_cast<uint64_t *>(tw_s + kPrimes * N);
+  uint64_t *acc = acc_all + comp * N;
+  uint32_t *xb = reinterpret_cast<uint32_t *>(acc_all + 2 * N) + group * B::XB_WORDS;
+  uint4 *part = reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(acc_all + 2 * N) + B::GROUPS * B::XB_WORDS);
+  uint32_t *res = reinterpret_cast<uint32_t *>(part + B::GROUPS * 2 * T);
+  uint16_t *atil = reinterpret_cast<uint16_t *>(res + 8 * N);
+
+  const uint32_t p = a.cc.pr[q].p, p_inv = a.cc.pr[q].p_inv;
+  const NttPrime npr(a.cc.pr[q]);
+  const uint32_t level = LEV > 0 ? static_cast<uint32_t>(LEV) : a.level;
+
+  for (uint32_t m = threadIdx.x; m < kPrimes * N; m += B::THREADS)
+    tw_s[m / N * N + split_tw_slot<LOGN>(m % N)] = a.tw[m];
+  const SplitTw<LOGN, 3> tw{tw_s + q * N, a.tw_lo[q]};
+  const uint64_t *lwe = a.lwe_in + static_cast<size_t>((a.lwe_first + ct) % a.lwe_count) * (a.n + 1);
+  constexpr uint32_t SH = 63 - LOGN;  // 64 - log2(2N)
+  for (uint32_t i = threadIdx.x; i <= a.n; i += B::THREADS)
+    atil[i] = static_cast<uint16_t>(((lwe[i] + (1ull << (SH - 1))) >> SH) & (TWO_N - 1));
+  __syncthreads();
+  {
+    const uint32_t btil = atil[a.n];
+    uint32_t li = 0;
+    if (!a.glwe_in && a.lut_index) {
+      li = a.lut_index[ct];
+      if (li >= a.num_luts) {  // never read outside the LUT array
+        if (threadIdx.x == 0 && a.err_flag) atomicExch(a.err_flag, 1u);
+        li = 0;
+      }
+    }
+    for (uint32_t m = threadIdx.x; m < 2 * N; m += B::THREADS) {
+      const uint32_t c = m / N, j = m % N, e = (j + btil) & (TWO_N - 1), t = e & (N - 1);
+      uint64_t v;
+      if (a.glwe_in) {
+        // encrypted test polynomial: ACC = X^{-b~} (A, B) for this ciphertext
+        v = a.glwe_in[(static_cast<size_t>(ct) * 2 + c) * N + t];
+      } else {
+        // trivial GLWE (0, X^{-b~} v): (X^{2N - b~} v)[j] = +-v[t], t = (j + b~) mod 2N folded into [0, N)
+        const uint64_t *lut = a.lut + (static_cast<size_t>(li) << a.msg_bits);
+        const uint32_t box = N >> a.msg_bits, h = box >> 1;
+        v = c == 0 ? 0ull : ((t < N - h) ? lut[(t + h) / box] : (0ull - lut[0]));
+      }
+      acc_all[m] = e >= N ? 0ull - v : v;
+    }
+  }
+  __syncthreads();
+
+  const uint64_t dig_add = dig_offset(a.base_log, level);
+  const uint32_t dig_bias = p - (1u << (a.base_log - 1));
+  const size_t kblk = static_cast<size_t>(2 * level) * 2 * N;  // words of one step's key block per prime
+  const uint32_t *key_own = a.bsk + q * kblk + (static_cast<size_t>(comp) * level * 2 + comp) * N + E * tau;
+  const uint32_t *key_oth = a.bsk + q * kblk + (static_cast<size_t>(comp) * level * 2 + (comp ^ 1u)) * N + E * tau;
+  const auto step_off = [&](uint32_t i) { return static_cast<size_t>(i) * kPrimes * kblk; };
+  const auto key_ok = [&](uint32_t i) {
+    return dbg_ok(a.bsk_words == 0 || (static_cast<size_t>(i) * kPrimes + q + 1) * kblk <= a.bsk_words, a.err_flag);
+  };
+  RowKeys<2> key;  // of the first rows of the coming step
+  const auto load_first = [&](uint32_t i) {
+    key.load(key_own + step_off(i), key_oth + step_off(i), 2 * N, key_ok(i), level);
+  };
+  const auto next_step = [&](uint32_t i) {
+    while (i < a.n && atil[i] == 0) ++i;
+    return i;
+  };
+  uint32_t i = next_step(0);
+  if (i < a.n) load_first(i);
+#pragma unroll 1
+  while (i < a.n) {
+    const uint32_t at = atil[i];
+    // ---- rotated difference of component comp, digit offsets added ----
+    uint64_t w[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const uint32_t j = tau + e * T, t = (j + TWO_N - at) & (TWO_N - 1);
+      const uint64_t v = acc[t & (N - 1)];
+      w[e] = (t >= N ? 0ull - v : v) - acc[j] + dig_add;
+    }
+    const uint32_t next = next_step(i + 1);
+
+    // ---- forward transforms, products with both components of the key ----
+    uint32_t own[E], oth[E];
+#pragma unroll
+    for (uint32_t lev = 0; lev < level; lev += 2) {
+      if (lev > 0)
+        key.load(key_own + step_off(i) + lev * 2 * N, key_oth + step_off(i) + lev * 2 * N, 2 * N, key_ok(i),
+                 level - lev);
+      uint32_t x[2][E];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          x[r][e] = lev + r < level ? biased_digit(w[e], a.base_log, lev + r) + dig_bias : p;
+      ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, npr, pairs);
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[r][e] = cond_sub(x[r][e], npr.p8);
+      mac<false, 2>(oth, x, key, 1, lev == 0, p, p_inv);
+      mac<false, 2>(own, x, key, 0, lev == 0, p, p_inv);
+    }
+    if (next < a.n) load_first(next);
+    part[(group ^ 1u) * 2 * T + tau] = make_uint4(oth[0], oth[1], oth[2], oth[3]);
+    part[(group ^ 1u) * 2 * T + T + tau] = make_uint4(oth[4], oth[5], oth[6], oth[7]);
+    __syncthreads();  // partial products there (and the exchange buffer free to change layout)
+    const uint4 pa = part[group * 2 * T + tau], pb = part[group * 2 * T + T + tau];
+    const uint32_t got[E] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+    uint32_t y[1][E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) y[0][e] = cond_sub(own[e] + got[e], 4 * p);  // both below 4p
+    ntt_inverse<LOGN, E, 1, 1>(y, tw, xb, tau, npr, singles);  // CRT-scaled through the keys
+
+    // ---- explicit CRT: group (q, comp) takes slots 2q and 2q + 1 of its component ----
+#pragma unroll
+    for (int e = 0; e < E; ++e) res[(q * 2 + comp) * N + e * T + tau] = y[0][e];
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t j = (2 * q + h) * T + tau;
+      uint64_t s = acc[j];
+      uint32_t ysum = 0;
+#pragma unroll
+      for (int k = 0; k < kPrimes; ++k) {
+        const uint32_t yv = res[(k * 2 + comp) * N + j];
+        s += static_cast<uint64_t>(yv) * a.cc.pr[k].Mp_mod64;
+        ysum += yv >> 2;
+      }
+      acc[j] = s - static_cast<uint64_t>(crt_quotient(ysum)) * a.cc.M_mod64;
+    }
+    i = next;
+    __syncthreads();
+  }
+
+  if (a.glwe_out) {
+    // ---- the rotated accumulator itself ----
+    uint64_t *gout = a.glwe_out + static_cast<size_t>(ct) * 2 * N;
+    for (uint32_t m = threadIdx.x; m < 2 * N; m += B::THREADS) gout[m] = acc_all[m];
+  } else {
+    // ---- sample extraction of the constant coefficient ----
+    uint64_t *out = a.lwe_big_out + static_cast<size_t>(ct) * (N + 1);
+    for (uint32_t j = threadIdx.x; j < N; j += B::THREADS) out[j == 0 ? 0 : N - j] = j == 0 ? acc_all[j] : 0ull - acc_all[j];
+    if (threadIdx.x == 0) out[N] = acc_all[N];
+  }
+}
+
+template <int LEV>
+static cudaError_t launch_brt_t(const BrArgs &a, cudaStream_t s) {
+  auto kern = blind_rotate_tiny_kernel<LEV>;
+  const size_t smem = br_tiny_smem_bytes(a.n);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e != cudaSuccess) return e;
+  kern<<<a.batch, BrtShape::THREADS, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_blind_rotate_tiny(const BrArgs &a, cudaStream_t s) {
+  return a.level == 2 ? launch_brt_t<2>(a, s) : launch_brt_t<0>(a, s);
+}
+
 bool br_small_supported(uint32_t logN, uint32_t level, uint32_t primes) {
   if (primes == kPrimes31) return logN == 12 && level >= 1 && level <= 3;
   return logN >= 8 && (logN <= 10 || (logN == 11 && level >= 1 && level <= 2));

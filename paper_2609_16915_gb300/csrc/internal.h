@@ -147,6 +147,8 @@ cudaError_t launch_blind_rotate_solo(const BrArgs &a, uint32_t workers, cudaStre
 // small batches (blind_rotate_small.cu): two CTAs per prime, one per component
 bool br_small_supported(uint32_t logN, uint32_t level, uint32_t primes);
 size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes);
+size_t br_tiny_smem_bytes(uint32_t n);  // N = 256, four primes: one CTA per ciphertext, any level
+cudaError_t launch_blind_rotate_tiny(const BrArgs &a, cudaStream_t s);
 cudaError_t launch_blind_rotate_small(const BrArgs &a, uint32_t logN, cudaStream_t s);
 // a.primes selects the kernel: the four-prime one or the three-prime one
 cudaError_t launch_blind_rotate(const BrArgs &a, uint32_t logN, bool dig16, cudaStream_t s);

@@ -365,6 +365,9 @@ struct GroupThreads {
   uint32_t id, threads;
   __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 };
+struct GroupSingles : GroupThreads {  // the same threads, single words
+  static constexpr bool kPairs = false;
+};
 
 template <int G, int WARPS, class TH>
 __device__ __forceinline__ void group_sync(uint32_t tau, const TH &th) {

@@ -295,16 +295,20 @@ BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) 
 // at the smaller rings while its CTAs of one or two warps do not crowd the SMs.
 // Measured against the cluster kernels as they were then: N = 2048, n = 742: 1
 // ciphertext 2.54 ms against 3.78, 15: 2.57 / 3.50, 16: 4.14 / 3.50; N = 4096, n = 840: 1: 6.3 / 10.7,
-// 22: 6.0 / 9.8, 24: 12.0 / 9.8; N = 256, n = 64: 16: 145 us / 257, 128: 194 / 267,
-// 256: 359 / 333; N = 512, n = 64: 8: 283 / 578, 100: 550 / 750, 200: 1064 / 980.
+// 22: 6.0 / 9.8, 24: 12.0 / 9.8; N = 512, n = 64: 8: 283 us / 578, 100: 550 / 750, 200: 1064 / 980.
+// N = 256, n = 64, against its kernel of one CTA per ciphertext, with the key
+// switch: 16: 135 us / 166, 64: 142 / 170, 76: 175 / 170 (a second cluster on an SM's
+// slots), 152: 312 / 173.
 static uint32_t br_small_max(const rosetta_ctx *c) {
   const uint32_t S = c->sms;
   if (c->br_primes == kPrimes31) return c->logN == 12 ? S * 3 / 20 : 0;
-  return c->logN <= 9 ? S * 3 / 4 : c->logN == 10 ? S / 5 : S / 10;
+  if (c->logN == 8) return S * 7 / 16;
+  return c->logN == 9 ? S * 3 / 4 : c->logN == 10 ? S / 5 : S / 10;
 }
 
-// Blind rotation of a batch: the small-batch kernel, the cluster kernels, or at
-// the standard ring, where the context holds the float quotient's key, one worker per ciphertext for
+// Blind rotation of a batch: the small-batch kernel, the cluster kernels (at N = 256
+// the kernel of one CTA per ciphertext, which takes at most 47 KB + 2 n bytes of shared
+// memory and so holds every accepted n), or at the standard ring, where the context holds the float quotient's key, one worker per ciphertext for
 // whatever part of the batch fills the GPU.  A launch of w workers per SM takes
 // the same time for any number of ciphertexts up to w S (S SMs; measured at
 // n = 742, with the key switch: 8.6, 13.4, 19.1 ms for w = 1, 2, 3), the cluster
@@ -314,8 +318,8 @@ static uint32_t br_small_max(const rosetta_ctx *c) {
 // is still ahead: r <= 3/4 S and S < r <= 5/4 S.
 cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t s) {
   const auto cluster = [&](const BrArgs &b) {
-    return c->br_small && b.batch <= br_small_max(c) ? launch_blind_rotate_small(b, c->logN, s)
-                                                     : launch_blind_rotate(b, c->logN, c->dig16, s);
+    if (c->br_small && b.batch <= br_small_max(c)) return launch_blind_rotate_small(b, c->logN, s);
+    return c->logN == 8 ? launch_blind_rotate_tiny(b, s) : launch_blind_rotate(b, c->logN, c->dig16, s);
   };
   if (!c->br_qf) return cluster(a);
   const uint32_t S = c->sms, wave = 3 * S;

@@ -11,9 +11,10 @@
 // is recombined in the epilogue.  Same words as keyswitch_kernel.
 //
 // Measured: n = 742, N = 2048, base 2^3 x 5, 4096 ciphertexts: 668 us with the
-// bf16 kernel, 271 here (the tensor floor is 208); n = 840, N = 4096, base 2^4 x 5,
-// 61 ciphertexts: 358 us with the CUDA-core kernel, 50 here (225 MB of limbs: 33).
-// So it takes every batch.
+// bf16 kernel, 262 here (the tensor floor is 208); n = 840, N = 4096, base 2^4 x 5,
+// 61 ciphertexts: 355 us with the CUDA-core kernel, 47 here (225 MB of limbs: 33).
+// So it takes every batch.  The main kernel starts while the digits are cut
+// (programmatic launch) and fetches its first key tiles meanwhile: 271 and 51 us without.
 //
 // Against the bf16 kernel (keyswitch_tc.cu: 8 limbs of 8 bits, or 16 of 4 bits
 // for long sums, at half the rate and two bytes each) a key word takes 13 bytes
@@ -90,6 +91,9 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// The digits (and the zeroed output) of the kernel before this one are complete.
+__device__ __forceinline__ void digits_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <int MT>
 struct F8Shape {
   static constexpr uint32_t STAGE = MT * F8_A_TILE + F8_B_TILE;
@@ -107,6 +111,8 @@ __global__ void __launch_bounds__(256) ks8_digits_kernel(const uint64_t *__restr
                                                          uint32_t batch, uint32_t kN, uint32_t base_log, uint32_t level,
                                                          uint32_t k_steps, uint64_t offset, uint64_t *__restrict__ zero,
                                                          size_t zero_words) {
+  // ks8_kernel may start: it sets itself up and fetches key tiles until these digits are complete
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // (the output, when K is split: the sums are added into it)
   const size_t gid = (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
   for (size_t w = gid; w < zero_words; w += static_cast<size_t>(gridDim.x) * gridDim.y * blockDim.x) zero[w] = 0;
@@ -216,18 +222,27 @@ __global__ void __launch_bounds__(F8_THREADS, 1) ks8_kernel(const KsTcArgs a) {
     uint32_t stage_bytes = F8_B_TILE, k = 0;
 #pragma unroll
     for (int m = 0; m < MT; ++m) stage_bytes += a_bytes[m];
+    const auto load_key = [&](uint32_t k) {
+      const uint32_t slot = k % STAGES;
+      expect_tx(full(slot), stage_bytes);
+      bulk_load(base + slot * S::STAGE + MT * F8_A_TILE, b8 + (static_cast<size_t>(nt) * a.k_steps + k0 + k) * F8_B_TILE,
+                F8_B_TILE, full(slot));
+    };
+    // the first stages' key tiles do not depend on the digits kernel
+    const uint32_t early = min(steps, STAGES);
+    for (uint32_t e = 0; e < early; ++e) load_key(e);
+    digits_ready();
     for (; k < steps; ++k) {
       const uint32_t slot = k % STAGES;
-      if (k >= STAGES && !mbar_wait(empty(slot), (k / STAGES - 1) & 1u)) break;  // the MMAs reading the slot are done
-      expect_tx(full(slot), stage_bytes);
-      const uint32_t dst = base + slot * S::STAGE;
+      if (k >= STAGES) {
+        if (!mbar_wait(empty(slot), (k / STAGES - 1) & 1u)) break;  // the MMAs reading the slot are done
+        load_key(k);
+      }
 #pragma unroll
       for (int m = 0; m < MT; ++m)
         if (a_bytes[m])
-          bulk_load(dst + m * F8_A_TILE, a8 + (static_cast<size_t>(mt * MT + m) * a.k_steps + k0 + k) * F8_A_TILE,
-                    a_bytes[m], full(slot));
-      bulk_load(dst + MT * F8_A_TILE, b8 + (static_cast<size_t>(nt) * a.k_steps + k0 + k) * F8_B_TILE, F8_B_TILE,
-                full(slot));
+          bulk_load(base + slot * S::STAGE + m * F8_A_TILE,
+                    a8 + (static_cast<size_t>(mt * MT + m) * a.k_steps + k0 + k) * F8_A_TILE, a_bytes[m], full(slot));
     }
     s_issued = k;
     if (k < steps) {
@@ -277,6 +292,7 @@ __global__ void __launch_bounds__(F8_THREADS, 1) ks8_kernel(const KsTcArgs a) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
   if (!unsafe && !partial && warp < 4) {
+    digits_ready();  // (long since; orders the output's zeros before the additions below)
     // epilogue: lane = ciphertext row of this warp's quarter of tensor memory
     const uint32_t n1 = a.n + 1, j0 = nt * F8_WORDS;
 #pragma unroll 1
@@ -348,8 +364,17 @@ static cudaError_t launch_ks8_t(const KsTcArgs &a, dim3 grid, cudaStream_t s) {
   const int smem = static_cast<int>(F8Shape<MT>::STAGES * F8Shape<MT>::STAGE);
   cudaError_t e = cudaFuncSetAttribute(ks8_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  ks8_kernel<MT><<<grid, F8_THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(F8_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, ks8_kernel<MT>, a);
 }
 
 cudaError_t launch_keyswitch_fp8(const KsTcArgs &a, uint32_t base_log, uint32_t level, uint32_t sms, cudaStream_t s) {

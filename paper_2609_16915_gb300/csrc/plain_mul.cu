@@ -51,7 +51,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
 #pragma unroll 1
   for (uint32_t q = 0; q < kPrimes; ++q) {
     const uint32_t p = a.cc.pr[q].p, p_inv = a.cc.pr[q].p_inv;
-  const NttPrime np(a.cc.pr[q]);
+    const NttPrime np(a.cc.pr[q]);
     // digit u - 2^31 mod p: u = (u >> 28) 2^28 + .., 2^28 = p + g with g < 2^18;
     // 2^31 = 8p + 8g
     const uint32_t bias = p - 8 * ((1u << 28) - p);

@@ -35,6 +35,8 @@ __global__ void __launch_bounds__((1 << LOGN) / 8)
   const uint32_t q = blockIdx.y;
   const PrimeConsts pc = cc.pr[q];
   const uint32_t p = pc.p;
+  // a plaintext product launched behind this one may start on its ciphertexts
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (uint32_t m = tau; m < N; m += T) tw[m] = tw_all[q * N + m];
 
   const uint64_t *src = raw + static_cast<size_t>(poly) * N;

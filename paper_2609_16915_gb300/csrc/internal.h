@@ -105,6 +105,7 @@ struct PlainMulArgs {
   const uint32_t *keys;       // transform domain [polys][prime][2][N]
   const uint64_t *plain_add;  // Q [polys][N], or null
   uint32_t batch, polys;
+  bool key_pending;           // launched right behind the transform of `keys` (and of nothing else it reads)
   const uint2 *tw;            // [prime][N]
   uint2 tw_lo[kPrimes][8];
   CrtConsts cc;

@@ -14,10 +14,14 @@
 // words are read and written once, straight between global memory and registers,
 // and nothing but the exchanges crosses threads.  The twiddles of one prime at a
 // time lie in shared memory.  80 registers: 24 warps per SM at N = 2048.
+// Launched behind the transform of its rows (rosetta_plaintext_mul_batch) it starts
+// while that runs and waits for it only before the first product.
 // Measured, N = 2048, 512 ciphertexts, the whole call with its host-side rows:
 // 198 us with the trace kernel's one-step mode (base 2^16 digits, eight rows whose
 // cross-component half was zero); 111 with one CTA of 128 registers for both
-// components (71 us of it the kernel: 1.7 waves of long CTAs); 107 here (64 us the kernel, bound by its transforms).
+// components (71 us of it the kernel: 1.7 waves of long CTAs); 100 with these (64 us
+// the kernel, 2.2 waves at the transforms' own rate of 10 butterflies per clock
+// and SM); 95 with the early start.
 #include <stdint.h>
 
 #include "internal.h"
@@ -25,8 +29,16 @@
 
 namespace rosetta {
 
+// Words that the kernel before this one may still be writing when this one starts:
+// an ordinary load that stays behind the wait (a read-only one, __ldg, may be moved before it).
+__device__ __forceinline__ uint4 ld_row(const uint4 *p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 template <int LOGN>
-__global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >> LOGN))
+__global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : LOGN == 8 ? 20 : 3 * (2048 >> LOGN))
     plain_mul_kernel(const __grid_constant__ PlainMulArgs a) {
   constexpr uint32_t N = 1u << LOGN, T = N / 8;
   constexpr int E = 8;
@@ -67,11 +79,12 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN >= 12 ? 1 : 3 * (2048 >>
       x[1][e] = cond_sub(lo - (lo >> 28) * p, p) + bias;
     }
     ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, np, CtaPairs());
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the plaintext's rows are there (key_pending)
     const uint4 *g = reinterpret_cast<const uint4 *>(a.keys + (static_cast<size_t>(which) * kPrimes + q) * 2 * N + E * tau);
     uint32_t o[1][E];
 #pragma unroll
     for (int k = 0; k < E / 4; ++k) {
-      const uint4 v0 = __ldg(g + k), v1 = __ldg(g + N / 4 + k);
+      const uint4 v0 = ld_row(g + k), v1 = ld_row(g + N / 4 + k);
       const uint32_t k0[4] = {v0.x, v0.y, v0.z, v0.w}, k1[4] = {v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
@@ -106,8 +119,17 @@ static cudaError_t launch_pm_t(const PlainMulArgs &a, cudaStream_t s) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  kern<<<2 * a.batch * a.polys, N / 8, smem, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * a.batch * a.polys, 1, 1);
+  cfg.blockDim = dim3(N / 8, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.key_pending ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
 cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, cudaStream_t s) {

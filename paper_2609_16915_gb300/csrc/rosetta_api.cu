@@ -253,7 +253,7 @@ void small_tables(const rosetta_ctx *c, Args *a) {
 // out[i][b] = (P_i * in_A, P_i * in_B + add_i) with P_i, i < polys, given by their
 // transformed rows.
 cudaError_t launch_pm(const rosetta_ctx *c, const uint32_t *key, const uint64_t *add, const uint64_t *in,
-                      uint32_t batch, uint64_t *out, cudaStream_t s, uint32_t polys = 1) {
+                      uint32_t batch, uint64_t *out, cudaStream_t s, uint32_t polys = 1, bool key_pending = false) {
   PlainMulArgs a{};
   a.glwe_in = in;
   a.glwe_out = out;
@@ -261,6 +261,7 @@ cudaError_t launch_pm(const rosetta_ctx *c, const uint32_t *key, const uint64_t 
   a.plain_add = add;
   a.batch = batch;
   a.polys = polys;
+  a.key_pending = key_pending;
   small_tables(c, &a);
   return launch_plaintext_mul(a, c->logN, s);
 }
@@ -744,7 +745,7 @@ int rosetta_plaintext_mul_batch(rosetta_ctx *c, const uint64_t *glwe_in, uint32_
   if (e == cudaSuccess && plain_add && !add_host)
     e = cudaMemcpyAsync(d_add, plain_add, N * 8, cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = launch_key_transform(c->d_pm_raw, c->d_pm_key, c->d_tw, c->cc, c->logN, 1, 1, s);
-  if (e == cudaSuccess) e = launch_pm(c, c->d_pm_key, plain_add ? d_add : nullptr, glwe_in, batch, glwe_out, s);
+  if (e == cudaSuccess) e = launch_pm(c, c->d_pm_key, plain_add ? d_add : nullptr, glwe_in, batch, glwe_out, s, 1, true);
   if (e != cudaSuccess) return cuda_fail(e);
   e = cudaStreamSynchronize(s);  // the host staging vector goes out of scope
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);

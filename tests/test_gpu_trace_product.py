@@ -63,3 +63,20 @@ def test_plaintext_product_at_the_ends_of_the_range(N):
         ctx.plaintext_mul_batch(G.to_dev(glwe), P.astype(np.int64), out, q)
         assert np.array_equal(G.to_host(out), O.plaintext_mul_batch(glwe, P, q))
     ctx.close()
+
+
+@pytest.mark.parametrize("N,batch", [(256, 1), (512, 40), (2048, 1), (2048, 400), (4096, 90)])
+def test_each_product_takes_its_own_plaintext(N, batch):
+    """Calls one after the other on the same buffers: a product kernel starts before
+    its plaintext is transformed and must not meet the rows of the call before."""
+    g = np.random.default_rng(N + batch)
+    glwe = g.integers(0, 2**64, size=(batch, 2, N), dtype=np.uint64)
+    pick = sorted({0, batch // 2, batch - 1})
+    ctx = _ctx(N)
+    d_in, out = G.to_dev(glwe), G.empty_dev(batch, 2, N)
+    for _ in range(4):
+        P = g.integers(-(1 << 40), 1 << 40, N)
+        q = g.integers(0, 2**64, size=N, dtype=np.uint64)
+        ctx.plaintext_mul_batch(d_in, P, out, q)
+        assert np.array_equal(G.to_host(out[pick]), O.plaintext_mul_batch(glwe[pick], P, q))
+    ctx.close()

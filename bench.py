@@ -136,13 +136,20 @@ def br_launches(p, batch, sms) -> int:
     return 2
 
 
+def trace_launches(p, batch, sms) -> int:
+    """Trace kernels of one call (gadget 2^16 x 4), as run_trace splits it."""
+    full, rest = divmod(batch, 3 * sms)
+    return 2 if br_solo(p) and full and 0 < rest <= 2 * sms + sms // 4 else 1
+
+
 def lookup_launches(p, batch, n_seg, sms) -> int:
     """Kernels of one segmented lookup: the segments go in groups of up to 4096
     ciphertexts (product, rotation, trace, accumulation each), with one product
     and rotation before and one product, rotation and trace after."""
     group = min(n_seg, max(1, 4096 // batch))
     sizes = [min(group, n_seg - s) for s in range(0, n_seg, group)]
-    return 5 + 2 * br_launches(p, batch, sms) + sum(3 + br_launches(p, m * batch, sms) for m in sizes)
+    each = [2 + br_launches(p, m * batch, sms) + trace_launches(p, m * batch, sms) for m in sizes]
+    return 4 + 2 * br_launches(p, batch, sms) + trace_launches(p, batch, sms) + sum(each)
 
 
 def ks_fp8(p) -> bool:

@@ -19,7 +19,7 @@ DEBUG_LIB = os.path.join(HERE, "librosetta_debug.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 SOURCES = ["tables.cu", "bsk_transform.cu", "blind_rotate.cu", "blind_rotate3.cu", "blind_rotate_solo.cu", "blind_rotate_small.cu",
            "keyswitch.cu", "keyswitch_tc.cu", "keyswitch_fp8.cu",
-           "rosetta_api.cu", "pbs_noalloc.cu", "trace.cu", "plain_mul.cu"]
+           "rosetta_api.cu", "pbs_noalloc.cu", "trace.cu", "trace_solo.cu", "plain_mul.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1,6 +1,6 @@
 // Single-precision complex transforms that estimate an external product's
-// size: the fourth CTA of a blind-rotation cluster runs them in place of a
-// fourth prime's number-theoretic transforms.
+// size: the worker-per-ciphertext kernels (blind_rotate_solo.cu, trace_solo.cu) run
+// them in place of a fourth prime's number-theoretic transforms.
 //
 // A real polynomial a(X) of N coefficients, multiplied modulo X^N + 1, is
 // carried as the complex polynomial sum_j (a_j + i a_{j+C}) X^j modulo

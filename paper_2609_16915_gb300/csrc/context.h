@@ -54,6 +54,8 @@ struct rosetta_ctx {
   uint64_t *d_lut = nullptr;      // staging for a host LUT  [2^p]
   uint32_t *d_err = nullptr;      // device-side argument error flag (LUT index out of range)
   uint32_t *d_trk = nullptr;      // trace automorphism keys, transform domain
+  uint32_t *d_trk_qf = nullptr;   // the same for the float quotient (trk_qf: for the present keys)
+  bool trk_qf = false;
   uint32_t trk_base_log = 0, trk_level = 0;
   bool have_trk = false;
   uint64_t *d_pm_raw = nullptr;   // plaintext-multiply rows P 2^32 and P, raw [2][N], and the additive plaintext [N]

@@ -93,7 +93,7 @@ struct TraceArgs {
   const uint32_t *keys;     // transform domain [steps][prime][level][2][N]
   const uint2 *tw;          // [prime][N]
   uint32_t base_log, level, batch;
-  uint2 tw_lo[kPrimes][8];  // each prime's first twiddles again, for the constant bank
+  uint2 tw_lo[kPrimes][kTwLo];  // each prime's first twiddles again, for the constant bank
   CrtConsts cc;
 };
 
@@ -170,6 +170,10 @@ cudaError_t launch_key_transform(const uint64_t *raw, uint32_t *out, const uint2
                                  uint32_t logN, uint32_t count, uint32_t rows, cudaStream_t s,
                                  uint32_t primes = kPrimes);
 cudaError_t launch_trace(const TraceArgs &a, uint32_t logN, cudaStream_t s);
+// the same for N = 2048 by one worker per ciphertext, `workers` per SM (trace_solo.cu);
+// keys [steps][3 primes + float][level][2][N]
+bool trace_solo_supported(uint32_t logN, uint32_t base_log, uint32_t level);
+cudaError_t launch_trace_solo(const TraceArgs &a, uint32_t workers, cudaStream_t s);
 cudaError_t launch_plaintext_mul(const PlainMulArgs &a, uint32_t logN, cudaStream_t s);
 // R (+)= sum_i X^(e0 + i step) r_i for i < polys: r [polys][count][N], R [count][N]
 cudaError_t launch_monomial_acc(uint64_t *R, const uint64_t *r, uint32_t count, uint32_t logN, uint32_t polys, uint32_t e0,

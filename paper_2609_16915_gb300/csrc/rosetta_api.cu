@@ -278,6 +278,41 @@ TraceArgs trace_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, u
   return a;
 }
 
+// Trace of a batch: clusters, or where the context holds the float quotient's trace
+// key one worker per ciphertext for whatever part of the batch fills the GPU.  A
+// launch of w workers per SM takes the same time for any number of ciphertexts up
+// to w S (S SMs; measured at gadget 2^16 x 4: 240, 362, 480 us for w = 1, 2, 3), the
+// cluster kernel about 42 us + 1.24 a ciphertext (152: 226, 228: 323, 304: 419, 456:
+// 603).  So whole waves of 3 S go to three workers, and of the rest r those up to
+// 5/3 S and from 2 S to 9/4 S to clusters, up to 2 S to two workers, more to three.
+cudaError_t run_trace(const rosetta_ctx *c, const TraceArgs &a, cudaStream_t s) {
+  if (!c->trk_qf) return launch_trace(a, c->logN, s);
+  const uint32_t S = c->sms, wave = 3 * S;
+  uint32_t full = a.batch / wave * wave, rest = a.batch - full;
+  if (rest > 2 * S + S / 4) {
+    full = a.batch;
+    rest = 0;
+  }
+  const auto slice = [&](uint32_t first, uint32_t count) {
+    TraceArgs t = a;
+    t.glwe_in += static_cast<size_t>(first) * 2 * c->prm.poly_size;
+    t.glwe_out += static_cast<size_t>(first) * 2 * c->prm.poly_size;
+    t.batch = count;
+    return t;
+  };
+  const auto solo = [&](uint32_t first, uint32_t count, uint32_t workers) {
+    TraceArgs t = slice(first, count);
+    t.keys = c->d_trk_qf;
+    t.tw = c->d_tw_qf;
+    t.cc = c->cc_qf;
+    return launch_trace_solo(t, workers, s);
+  };
+  cudaError_t e = full ? solo(0, full, 3) : cudaSuccess;
+  if (e != cudaSuccess || rest == 0) return e;
+  if (rest > S + S * 2 / 3 && rest <= 2 * S) return solo(full, rest, 2);
+  return launch_trace(slice(full, rest), c->logN, s);
+}
+
 // Ciphertexts [first, first + count) of a launch.
 BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) {
   a.lwe_first += first;
@@ -683,14 +718,19 @@ int rosetta_upload_trace_keys(rosetta_ctx *c, const uint64_t *keys, size_t n_wor
   }
   if (c->d_trk && c->trk_level != level) {
     cudaFree(c->d_trk);
-    c->d_trk = nullptr;
+    cudaFree(c->d_trk_qf);
+    c->d_trk = c->d_trk_qf = nullptr;
   }
+  const bool qf = c->br_qf && trace_solo_supported(c->logN, base_log, level);
   if (!c->d_trk) e = cudaMalloc(&c->d_trk, want * kPrimes * sizeof(uint32_t));
+  if (e == cudaSuccess && qf && !c->d_trk_qf) e = cudaMalloc(&c->d_trk_qf, want * kPrimes * sizeof(uint32_t));
   if (e != cudaSuccess) {
     if (tmp) cudaFreeAsync(tmp, s);
     return cuda_fail(e);
   }
   e = launch_key_transform(src, c->d_trk, c->d_tw, c->cc, c->logN, c->logN, level, s);
+  if (e == cudaSuccess && qf)
+    e = launch_bsk_transform_qf(src, c->d_trk_qf, c->d_tw_qf, c->d_tw_f64, c->cc_qf, c->logN, c->logN, level / 2, s);
   if (tmp) cudaFreeAsync(tmp, s);
   if (e != cudaSuccess) return cuda_fail(e);
   if (!src_is_device) {
@@ -699,6 +739,7 @@ int rosetta_upload_trace_keys(rosetta_ctx *c, const uint64_t *keys, size_t n_wor
   }
   c->trk_base_log = base_log;
   c->trk_level = level;
+  c->trk_qf = qf;
   c->have_trk = true;
   return ROSETTA_OK;
 }
@@ -713,7 +754,7 @@ int rosetta_trace_batch(rosetta_ctx *c, const uint64_t *glwe_in, uint32_t batch,
   if (!is_device_ptr(glwe_in) || !is_device_ptr(glwe_out) || !aligned8(glwe_in) || !aligned8(glwe_out) ||
       overlaps(glwe_in, gbytes, glwe_out, gbytes))
     return ROSETTA_ERR_INVALID_ARG;
-  cudaError_t e = launch_trace(trace_args(c, glwe_in, batch, glwe_out), c->logN, as_stream(stream));
+  cudaError_t e = run_trace(c, trace_args(c, glwe_in, batch, glwe_out), as_stream(stream));
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
 }
 
@@ -856,13 +897,13 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
     const uint32_t m = std::min(group, nseg - sg);
     e = launch_pm(c, c->d_lk_key + (1 + sg) * key_words, c->d_lk_add + (1 + sg) * N, glwe_x, batch, T, s, m);
     if (e == cudaSuccess) e = rotate(I, T, U, m * batch);
-    if (e == cudaSuccess) e = launch_trace(trace_args(c, U, m * batch, T), c->logN, s);
+    if (e == cudaSuccess) e = run_trace(c, trace_args(c, U, m * batch, T), s);
     if (e == cudaSuccess) e = launch_monomial_acc(R, T, 2 * batch, c->logN, m, sg * seg_box, seg_box, sg == 0, s);
   }
   // phase 2: spread each value over its segment box, rotate by [[S]], trace
   if (e == cudaSuccess) e = launch_pm(c, kBox, nullptr, R, batch, T, s);
   if (e == cudaSuccess) e = rotate(lwe_seg, T, U, batch);
-  if (e == cudaSuccess) e = launch_trace(trace_args(c, U, batch, glwe_out), c->logN, s);
+  if (e == cudaSuccess) e = run_trace(c, trace_args(c, U, batch, glwe_out), s);
   return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
 }
 
@@ -944,6 +985,7 @@ void rosetta_destroy(rosetta_ctx *c) {
   cudaFree(c->d_lut);
   cudaFree(c->d_err);
   cudaFree(c->d_trk);
+  cudaFree(c->d_trk_qf);
   cudaFree(c->d_pm_raw);
   cudaFree(c->d_pm_key);
   cudaFree(c->d_lk_key);

@@ -26,7 +26,8 @@
 // memory only, as in the blind rotation; the transforms exchange pairs; four
 // CTAs fit an SM at N = 2048.  Measured, N = 2048, gadget 2^16 x 4, 1024
 // ciphertexts: 1.84 ms with single-word exchanges, pushed residues and plain
-// barriers, 1.38 ms with these, 1.25 with 2p and 8p loaded as values (NttPrime).
+// barriers, 1.38 ms with these, 1.25 with 2p and 8p loaded as values (NttPrime).  At N = 2048
+// most of a large batch goes to trace_solo.cu.
 #include <cooperative_groups.h>
 
 #include "dsmem.cuh"

@@ -136,20 +136,28 @@ cudaError_t launch_keyswitch(const KsArgs &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// corr[o] = (B/2) * sum_rows ksk[row][o]  (mod 2^64)
-__global__ void ksk_corr_kernel(const uint64_t *__restrict__ ksk, uint64_t *__restrict__ corr, uint32_t rows,
+// corr[o] = (B/2) * sum_rows ksk[row][o]  (mod 2^64), the rows split over blockIdx.y
+// (one block of rows per column tile walks 10240 dependent loads at the standard set:
+// 742 us of the key's upload; 14 split).
+__global__ void ksk_corr_kernel(const uint64_t *__restrict__ ksk, unsigned long long *corr, uint32_t rows, uint32_t per,
                                 uint32_t n1, uint64_t half) {
   const uint32_t o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= n1) return;
+  const uint32_t r1 = min(rows, (blockIdx.y + 1) * per);
   uint64_t s = 0;
-  for (uint32_t r = 0; r < rows; ++r) s += ksk[static_cast<size_t>(r) * n1 + o];
-  corr[o] = s * half;
+#pragma unroll 4
+  for (uint32_t r = blockIdx.y * per; r < r1; ++r) s += ksk[static_cast<size_t>(r) * n1 + o];
+  atomicAdd(corr + o, static_cast<unsigned long long>(s * half));
 }
 
 cudaError_t launch_ksk_corr(const uint64_t *ksk, uint64_t *corr, uint32_t rows, uint32_t n, uint32_t base_log,
                             cudaStream_t s) {
-  const uint32_t n1 = n + 1;
-  ksk_corr_kernel<<<(n1 + 127) / 128, 128, 0, s>>>(ksk, corr, rows, n1, 1ull << (base_log - 1));
+  const uint32_t n1 = n + 1, per = 64;
+  cudaError_t e = cudaMemsetAsync(corr, 0, n1 * sizeof(uint64_t), s);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((n1 + 127) / 128, (rows + per - 1) / per);
+  ksk_corr_kernel<<<grid, 128, 0, s>>>(ksk, reinterpret_cast<unsigned long long *>(corr), rows, per, n1,
+                                       1ull << (base_log - 1));
   return cudaGetLastError();
 }
 

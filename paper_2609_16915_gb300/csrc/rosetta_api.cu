@@ -105,6 +105,15 @@ int ensure(uint64_t **buf, size_t *cap_words, size_t need, cudaStream_t s) {
   return ROSETTA_OK;
 }
 
+// Memory for the float quotient's second format of a key: without it the cluster
+// kernels take the work.
+bool try_malloc(uint32_t **buf, size_t bytes) {
+  if (cudaMalloc(reinterpret_cast<void **>(buf), bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  *buf = nullptr;
+  return false;
+}
+
 size_t lwe_words(const rosetta_ctx *c) { return c->prm.lwe_dim + 1; }
 size_t big_words(const rosetta_ctx *c) { return (size_t)c->prm.glwe_dim * c->prm.poly_size + 1; }
 size_t stage_words(const rosetta_ctx *c) { return big_words(c) > lwe_words(c) ? big_words(c) : lwe_words(c); }
@@ -519,7 +528,8 @@ int rosetta_upload_bsk(rosetta_ctx *c, const uint64_t *bsk, size_t n_words, int 
   // one 32-bit residue per prime of the blind rotation's set for every raw word
   const bool three = c->br_primes == kPrimes31;
   if (!c->d_bsk) e = cudaMalloc(&c->d_bsk, want * c->br_primes * sizeof(uint32_t));
-  if (e == cudaSuccess && c->br_qf && !c->d_bsk_qf) e = cudaMalloc(&c->d_bsk_qf, want * kPrimes * sizeof(uint32_t));
+  if (e == cudaSuccess && c->br_qf && !c->d_bsk_qf)
+    c->br_qf = try_malloc(&c->d_bsk_qf, want * kPrimes * sizeof(uint32_t));
   if (e != cudaSuccess) {
     if (tmp) cudaFreeAsync(tmp, s);
     return cuda_fail(e);
@@ -720,10 +730,12 @@ int rosetta_upload_trace_keys(rosetta_ctx *c, const uint64_t *keys, size_t n_wor
     cudaFree(c->d_trk);
     cudaFree(c->d_trk_qf);
     c->d_trk = c->d_trk_qf = nullptr;
+    c->have_trk = c->trk_qf = false;
+    c->trk_level = level;  // what the buffers are sized for from here on
   }
-  const bool qf = c->br_qf && trace_solo_supported(c->logN, base_log, level);
+  bool qf = c->br_qf && trace_solo_supported(c->logN, base_log, level);
   if (!c->d_trk) e = cudaMalloc(&c->d_trk, want * kPrimes * sizeof(uint32_t));
-  if (e == cudaSuccess && qf && !c->d_trk_qf) e = cudaMalloc(&c->d_trk_qf, want * kPrimes * sizeof(uint32_t));
+  if (e == cudaSuccess && qf && !c->d_trk_qf) qf = try_malloc(&c->d_trk_qf, want * kPrimes * sizeof(uint32_t));
   if (e != cudaSuccess) {
     if (tmp) cudaFreeAsync(tmp, s);
     return cuda_fail(e);
@@ -862,17 +874,23 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
   // (Where memory is too short for a group's scratch, one segment at a time.)
   // Measured, N = 2048, 4 segments: 256 lookups 82.3 -> 74.5 ms.
   uint32_t group = std::min(nseg, std::max(1u, 4096u / batch));
-  int r = ensure(&c->d_lk_t, &c->lk_t_cap, (size_t)group * batch * gw, s);
-  if (r == ROSETTA_OK) r = ensure(&c->d_lk_u, &c->lk_u_cap, (size_t)group * batch * gw, s);
+  const auto scratch = [&](size_t segments) {
+    int st = ensure(&c->d_lk_t, &c->lk_t_cap, segments * batch * gw, s);
+    if (st == ROSETTA_OK) st = ensure(&c->d_lk_u, &c->lk_u_cap, segments * batch * gw, s);
+    if (st == ROSETTA_OK) st = ensure(&c->d_lk_R, &c->lk_R_cap, batch * gw, s);
+    if (st == ROSETTA_OK) st = ensure(&c->d_lk_I, &c->lk_I_cap, batch * lwe_words(c), s);
+    return st == ROSETTA_OK ? ensure_big(c, batch, s) : st;
+  };
+  int r = scratch(group);
   if (r == ROSETTA_ERR_OOM && group > 1) {
     cudaGetLastError();
     group = 1;
-    r = ensure(&c->d_lk_t, &c->lk_t_cap, batch * gw, s);
-    if (r == ROSETTA_OK) r = ensure(&c->d_lk_u, &c->lk_u_cap, batch * gw, s);
+    if (c->d_lk_t) cudaFreeAsync(c->d_lk_t, s);
+    if (c->d_lk_u) cudaFreeAsync(c->d_lk_u, s);
+    c->d_lk_t = c->d_lk_u = nullptr;
+    c->lk_t_cap = c->lk_u_cap = 0;
+    r = scratch(1);
   }
-  if (r == ROSETTA_OK) r = ensure(&c->d_lk_R, &c->lk_R_cap, batch * gw, s);
-  if (r == ROSETTA_OK) r = ensure(&c->d_lk_I, &c->lk_I_cap, batch * lwe_words(c), s);
-  if (r == ROSETTA_OK) r = ensure_big(c, batch, s);
   if (r != ROSETTA_OK) return r;
   const size_t key_words = (size_t)kPrimes * gw;
   const uint32_t *kP = c->d_lk_key, *kBox = c->d_lk_key + (1 + nseg) * key_words;

@@ -82,7 +82,7 @@ struct BrShape {
   static constexpr int QE = E / 4;                     // first-pass slots per owner quarter
   static constexpr int XBUF = br_xbuf(LOGN);            // exchange buffers (polys)
   // resident CTAs per SM the register allocation must allow (shared memory
-  // allows the same: 4 x 46 KB at N = 2048, 2 x 90 KB at 4096)
+  // allows the same: 4 x 48.5 KB at N = 2048, 2 x 90 KB at 4096)
   static constexpr int MIN_CTAS = (LOGN <= 11) ? 4 : (LOGN == 12 ? 2 : 1);
 };
 

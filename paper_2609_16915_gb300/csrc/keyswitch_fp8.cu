@@ -106,7 +106,9 @@ struct F8Shape {
 // Digit tiles: A[b][r] = digit lev of a'_i (closed form, see biased_digit),
 // all levels of 128 mask words x 32 ciphertexts per CTA: a word is read once.  A
 // warp writes whole core matrices (8 rows x 16 bytes, 128 contiguous bytes).
-// Also zeroes `zero_words` words of the output.
+// Also zeroes `zero_words` words of the output.  The grid has one dimension, kN / 128
+// CTAs (at most 64) per 32 ciphertexts: its limit of 2^31 - 1 lies beyond any batch
+// that fits the memory, that of a second dimension (65535) does not.
 __global__ void __launch_bounds__(256) ks8_digits_kernel(const uint64_t *__restrict__ big, uint8_t *__restrict__ a_tiles,
                                                          uint32_t batch, uint32_t kN, uint32_t base_log, uint32_t level,
                                                          uint32_t k_steps, uint64_t offset, uint64_t *__restrict__ zero,
@@ -114,9 +116,10 @@ __global__ void __launch_bounds__(256) ks8_digits_kernel(const uint64_t *__restr
   // ks8_kernel may start: it sets itself up and fetches key tiles until these digits are complete
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // (the output, when K is split: the sums are added into it)
-  const size_t gid = (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
-  for (size_t w = gid; w < zero_words; w += static_cast<size_t>(gridDim.x) * gridDim.y * blockDim.x) zero[w] = 0;
-  const uint32_t i0 = blockIdx.x * F8_K, g0 = blockIdx.y * 4;  // first mask word, first group of 8 ciphertexts
+  const size_t gid = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (size_t w = gid; w < zero_words; w += static_cast<size_t>(gridDim.x) * blockDim.x) zero[w] = 0;
+  const uint32_t k_blocks = kN / F8_K, group = blockIdx.x / k_blocks;
+  const uint32_t i0 = (blockIdx.x - group * k_blocks) * F8_K, g0 = group * 4;  // first mask word, group of 8 ciphertexts
   const uint32_t warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const uint32_t r = lane >> 2, q = lane & 3u;  // row of the group, four of the core matrix's 16 words
   const int half = 1 << (base_log - 1);
@@ -396,7 +399,9 @@ cudaError_t launch_keyswitch_fp8(const KsTcArgs &a, uint32_t base_log, uint32_t 
       splits = z;
     }
   }
-  ks8_digits_kernel<<<dim3(a.kN / F8_K, (a.batch + 31) / 32), 256, 0, s>>>(
+  const uint64_t digit_ctas = static_cast<uint64_t>((a.batch + 31ull) / 32) * (a.kN / F8_K);
+  if (digit_ctas > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+  ks8_digits_kernel<<<static_cast<uint32_t>(digit_ctas), 256, 0, s>>>(
       a.big, reinterpret_cast<uint8_t *>(const_cast<uint16_t *>(a.a_tiles)), a.batch, a.kN, base_log, level, a.k_steps,
       offset, a.out, splits > 1 ? static_cast<size_t>(a.batch) * (a.n + 1) : 0);
   cudaError_t e = cudaGetLastError();

@@ -94,14 +94,16 @@ struct BrsShape {
 };
 
 __host__ __device__ constexpr size_t brs_smem(size_t N, bool single, size_t n, size_t primes) {
-  return (N * sizeof(uint2) + N * sizeof(uint64_t) + (single ? 1 : 2) * (N + N / 8) * sizeof(uint32_t) +
+  return (4 * sizeof(uint64_t) + N * sizeof(uint2) + N * sizeof(uint64_t) + (single ? 1 : 2) * (N + N / 8) * sizeof(uint32_t) +
           2 * N * sizeof(uint32_t) + 2 * (primes - 1) * N * sizeof(uint32_t) + (n + 1) * sizeof(uint16_t) + 15) & ~size_t(15);
 }
 
 }  // namespace
 
 // PRIMES: 4 (28-bit set) or 3 (31-bit set).  LEV > 0: levels known at compile
-// time; 0: from the arguments.  Shared memory: twiddles of prime q uint2 [N], acc
+// time; 0: from the arguments.  Shared memory, all of it dynamic, so that
+// brs_smem is the whole of what a CTA takes: mbarriers uint64 [4] (partial
+// products, residues of even steps; of odd ones), twiddles of prime q uint2 [N], acc
 // uint64 [N], exchange buffer, received partial products uint32 [2 steps][2][T][4], received
 // residues uint32 [2 steps][PRIMES - 1][2][T][4], switched mask and body uint16 [n+1].
 template <int LOGN, int LEV, int PRIMES>
@@ -120,10 +122,10 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
   if (!dbg_ok(ct < a.batch, a.err_flag)) return;  // the whole cluster shares ct
 
   extern __shared__ __align__(16) unsigned char smem[];
-  uint2 *tw_s = reinterpret_cast<uint2 *>(smem);
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
+  uint2 *tw_s = reinterpret_cast<uint2 *>(bars + 4);
   uint64_t *acc = reinterpret_cast<uint64_t *>(tw_s + N);
   uint32_t *xb = reinterpret_cast<uint32_t *>(acc + N);
-  __shared__ __align__(8) uint64_t bars[4];  // partial products, residues of even steps; of odd ones
   uint4 *part = reinterpret_cast<uint4 *>(xb + B::XB_WORDS);
   uint4 *res = part + 4 * T;
   uint16_t *atil = reinterpret_cast<uint16_t *>(res + 2 * (PRIMES - 1) * 2 * T);

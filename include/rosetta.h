@@ -316,6 +316,16 @@ int rosetta_selftest_wait_timeout(rosetta_ctx *ctx, uint32_t limit_us, void *str
  * Errors: INVALID_ARG, KEYS_MISSING, CUDA, OOM. */
 int rosetta_selftest_bounds(rosetta_ctx *ctx, void *stream);
 
+/* Self-test of what the small-batch blind rotation does when one of its bounded
+ * waits gives up, in a library compiled with -DROSETTA_DEBUG (no counterpart in
+ * the paper): rotates one ciphertext with one CTA keeping back the words of one step, the
+ * waits limited to about limit_us microseconds (1 .. 10^6).  Every CTA of the cluster
+ * gives up in turn, a step apart, and ends; rosetta_sync_status then returns TIMEOUT
+ * once and the context stays usable.  Needs the BSK.  Regular build, and sets
+ * without a small-batch kernel: UNSUPPORTED_PARAMS.  Errors: INVALID_ARG, KEYS_MISSING,
+ * CUDA, OOM. */
+int rosetta_selftest_lost_words(rosetta_ctx *ctx, uint32_t limit_us, void *stream);
+
 /* Wait for all work on `stream` and report any deferred execution error
  * (CUDA; TIMEOUT when a bounded wait of a tensor-core key switch or of the
  * small-batch blind rotation gave up;

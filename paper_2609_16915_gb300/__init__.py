@@ -27,7 +27,7 @@ EXPORTS = ("rosetta_params_init", "rosetta_upload_bsk", "rosetta_upload_ksk", "r
            "rosetta_blind_rotate_extract_batch", "rosetta_keyswitch_batch", "rosetta_pbs_batch_multi_lut",
            "rosetta_blind_rotate_glwe_batch", "rosetta_upload_trace_keys", "rosetta_trace_batch",
            "rosetta_plaintext_mul_batch", "rosetta_upload_lookup_table", "rosetta_segmented_lookup_batch",
-           "rosetta_selftest_wait_timeout", "rosetta_selftest_bounds",
+           "rosetta_selftest_wait_timeout", "rosetta_selftest_bounds", "rosetta_selftest_lost_words",
            "rosetta_pbs_batch_noalloc", "rosetta_ntt_primes",
            "rosetta_sync_status", "rosetta_destroy", "rosetta_status_string")
 
@@ -72,6 +72,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     L.rosetta_segmented_lookup_batch.argtypes = [vp, u64p, u64p, u32, u64p, vp]
     L.rosetta_selftest_wait_timeout.argtypes = [vp, u32, vp]
     L.rosetta_selftest_bounds.argtypes = [vp, vp]
+    L.rosetta_selftest_lost_words.argtypes = [vp, u32, vp]
     L.rosetta_ntt_primes.argtypes = [vp]
     L.rosetta_sync_status.argtypes = [vp, vp]
     L.rosetta_destroy.argtypes = [vp]
@@ -244,6 +245,13 @@ class Context:
         sync_status as BOUNDS); the regular build returns UNSUPPORTED_PARAMS."""
         _check("rosetta_selftest_bounds", load().rosetta_selftest_bounds(self._h, _stream(stream)))
 
+    def rosetta_selftest_lost_words(self, limit_us=10000, stream=None):
+        """Make the waits of a small-batch blind rotation give up in a
+        ROSETTA_DEBUG build (reported by sync_status as TIMEOUT); the regular
+        build returns UNSUPPORTED_PARAMS."""
+        _check("rosetta_selftest_lost_words",
+               load().rosetta_selftest_lost_words(self._h, limit_us, _stream(stream)))
+
     def rosetta_pbs_batch_noalloc(self, lwe_in, lut, lwe_out, stream=None):
         """rosetta_pbs_batch without any device allocation in the call (fixed
         in-library scratch; device buffers only, bounded batch)."""
@@ -277,5 +285,6 @@ class Context:
     segmented_lookup_batch = rosetta_segmented_lookup_batch
     selftest_wait_timeout = rosetta_selftest_wait_timeout
     selftest_bounds = rosetta_selftest_bounds
+    selftest_lost_words = rosetta_selftest_lost_words
     ntt_primes = rosetta_ntt_primes
     sync_status = rosetta_sync_status

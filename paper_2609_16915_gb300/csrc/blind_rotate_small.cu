@@ -25,8 +25,13 @@
 // most of a step); 2.85 with two CTAs per prime and two barriers; 2.54 with
 // st.async, 2.42 with 2p and 8p loaded as values (NttPrime).
 //
-// Every wait gives up after about two seconds and raises the error flag; the CTA
-// then runs on without waiting.
+// Every wait gives up after about two seconds and raises the error flag.  The CTA
+// then finishes the step with what it has, all threads leave the loop after it
+// (no further words are sent and no mbarrier is armed again), and nothing is written
+// out.  Its peers miss its words in the next step and leave the same way, so every CTA
+// comes to the cluster barrier at the end; the CTA that gave up then waits, with a limit,
+// for the words that were still on their way to it: the rest of its last step's and, a
+// step early, those of the next.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -94,7 +99,7 @@ struct BrsShape {
 };
 
 __host__ __device__ constexpr size_t brs_smem(size_t N, bool single, size_t n, size_t primes) {
-  return (4 * sizeof(uint64_t) + N * sizeof(uint2) + N * sizeof(uint64_t) + (single ? 1 : 2) * (N + N / 8) * sizeof(uint32_t) +
+  return (6 * sizeof(uint64_t) + N * sizeof(uint2) + N * sizeof(uint64_t) + (single ? 1 : 2) * (N + N / 8) * sizeof(uint32_t) +
           2 * N * sizeof(uint32_t) + 2 * (primes - 1) * N * sizeof(uint32_t) + (n + 1) * sizeof(uint16_t) + 15) & ~size_t(15);
 }
 
@@ -103,8 +108,9 @@ __host__ __device__ constexpr size_t brs_smem(size_t N, bool single, size_t n, s
 // PRIMES: 4 (28-bit set) or 3 (31-bit set).  LEV > 0: levels known at compile
 // time; 0: from the arguments.  Shared memory, all of it dynamic, so that
 // brs_smem is the whole of what a CTA takes: mbarriers uint64 [4] (partial
-// products, residues of even steps; of odd ones), twiddles of prime q uint2 [N], acc
-// uint64 [N], exchange buffer, received partial products uint32 [2 steps][2][T][4], received
+// products, residues of even steps; of odd ones), a word raised when a wait gives up (and
+// padding to 16 bytes), twiddles of prime q uint2 [N], acc uint64 [N], exchange buffer, received
+// partial products uint32 [2 steps][2][T][4], received
 // residues uint32 [2 steps][PRIMES - 1][2][T][4], switched mask and body uint16 [n+1].
 template <int LOGN, int LEV, int PRIMES>
 __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
@@ -113,6 +119,7 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
   constexpr uint32_t N = B::N, T = B::T, TWO_N = 2 * N;
   constexpr int E = 8;
   constexpr bool P31 = PRIMES == kPrimes31;
+  constexpr uint16_t kStopped = 0xFFFF;  // in place of a switched mask word (below 2N)
 
   cg::cluster_group cluster = cg::this_cluster();
   const uint32_t rank = cluster.block_rank();
@@ -123,7 +130,8 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
 
   extern __shared__ __align__(16) unsigned char smem[];
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
-  uint2 *tw_s = reinterpret_cast<uint2 *>(bars + 4);
+  volatile uint32_t *stop = reinterpret_cast<uint32_t *>(bars + 4);
+  uint2 *tw_s = reinterpret_cast<uint2 *>(bars + 6);
   uint64_t *acc = reinterpret_cast<uint64_t *>(tw_s + N);
   uint32_t *xb = reinterpret_cast<uint32_t *>(acc + N);
   uint4 *part = reinterpret_cast<uint4 *>(xb + B::XB_WORDS);
@@ -136,6 +144,7 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
   const uint32_t level = LEV > 0 ? static_cast<uint32_t>(LEV) : a.level;
 
   if (tau == 0) {
+    *stop = 0u;
     for (int b = 0; b < 4; ++b) mbar_init(smem_addr(&bars[b]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -184,13 +193,11 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
   const uint32_t dig_bias = p - (1u << (a.base_log - 1));
   const uint32_t bar0 = smem_addr(bars), part_s = smem_addr(part), res_s = smem_addr(res);
   const uint32_t part_to = dsmem_map(part_s + tau * 16u, rank ^ 1u), part_bar_to = dsmem_map(bar0, rank ^ 1u);
-  bool waiting = true;  // until a wait gives up
-  const auto wait = [&](uint32_t bar, uint32_t parity) {
-    if (!mbar_wait_cluster(bar, parity, waiting ? kWaitCycles : 0)) {
-      waiting = false;
-      if (a.err_flag) atomicExch(a.err_flag, 2u);
-    }
-  };
+#ifdef ROSETTA_DEBUG
+  const long long wait_cycles = a.wait_cycles ? a.wait_cycles : kWaitCycles;
+#else
+  constexpr long long wait_cycles = kWaitCycles;
+#endif
   const size_t kblk = static_cast<size_t>(2 * level) * 2 * N;  // words of one step's key block per prime
   // this thread's words of the first row of component comp, own and partner's column
   const uint32_t *key_own = a.bsk + q * kblk + (static_cast<size_t>(comp) * level * 2 + comp) * N + E * tau;
@@ -216,10 +223,10 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
     const uint32_t at = atil[i];
     const uint32_t odd = step & 1u, phase = (step >> 1) & 1u;
     const uint32_t part_bar = bar0 + 16u * odd, res_bar = part_bar + 8u;
-    if (tau == 0) {
-      expect_tx(part_bar, N * 4u);
-      expect_tx(res_bar, (PRIMES - 1) * N * 4u);
-    }
+    // A wait of the last step gave up: the same for all threads, as it was written before that
+    // step's last barrier and is not again before this one's first.  (The word is needed
+    // anyway; a flag of its own, or a barrier that reduces the threads', cost 1 to 3 %.)
+    if (at == kStopped) break;
     // ---- rotated difference, (X^a P)[j] = +-P[(j - a) mod 2N], digit offsets added ----
     uint64_t w[E];
 #pragma unroll
@@ -229,6 +236,17 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
       w[e] = (t >= N ? 0ull - v : v) - acc[j] + dig_add;
     }
     const uint32_t next = next_step(i + 1);
+    const auto wait = [&](uint32_t bar, uint32_t parity) {
+      if (!mbar_wait_cluster(bar, parity, wait_cycles)) {
+        *stop = 1u;
+        if (next < a.n) atil[next] = kStopped;
+        if (a.err_flag) atomicExch(a.err_flag, 2u);
+      }
+    };
+    if (tau == 0) {
+      expect_tx(part_bar, N * 4u);
+      expect_tx(res_bar, (PRIMES - 1) * N * 4u);
+    }
 
     // ---- forward transforms, products with both components of the key ----
     uint32_t own[E], oth[E];
@@ -252,6 +270,9 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
     };
     // the partner's half is on its way while the own half is multiplied
     const auto send = [&] {
+#ifdef ROSETTA_DEBUG
+      if (a.lose_step == step + 1 && rank == 0) return;  // (rosetta_selftest_lost_words)
+#endif
       const uint32_t to = part_to + odd * 2 * T * 16u, bar = part_bar_to + 16u * odd;
       dsmem_st_async_v4(to, oth[0], oth[1], oth[2], oth[3], bar);
       dsmem_st_async_v4(to + T * 16u, oth[4], oth[5], oth[6], oth[7], bar);
@@ -326,10 +347,13 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
     ++step;
     __syncthreads();
   }
+  const bool gave_up = *stop != 0u;  // in step - 1, the last that was run
 
   // the CTAs of a component all hold it: CTA (q, comp) writes its share
   const uint32_t j0 = N / PRIMES * q, j1 = q == PRIMES - 1 ? N : N / PRIMES * (q + 1);
-  if (a.glwe_out) {
+  if (gave_up) {
+    // the accumulator is not one of the ciphertext's
+  } else if (a.glwe_out) {
     // ---- the rotated accumulator itself ----
     uint64_t *gout = a.glwe_out + (static_cast<size_t>(ct) * 2 + comp) * N;
     for (uint32_t j = j0 + tau; j < j1; j += T) gout[j] = acc[j];
@@ -342,6 +366,22 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
       out[N] = acc[0];
   }
   cluster.sync();  // no CTA leaves while a peer may still store into it
+  if (gave_up && tau == 0) {
+    // Every store has been issued by now and takes microseconds to arrive.  The next
+    // step's mbarriers are armed here to count the early words: their phase before,
+    // the last step's but one, was complete when this step was run.
+    const auto arrived = [&](uint32_t st, bool arm) {
+      const uint32_t pb = bar0 + 16u * (st & 1u), ph = (st >> 1) & 1u;
+      if (arm) {
+        expect_tx(pb, N * 4u);
+        expect_tx(pb + 8u, (PRIMES - 1) * N * 4u);
+      }
+      mbar_wait_cluster(pb, ph, wait_cycles / 64);
+      mbar_wait_cluster(pb + 8u, ph, wait_cycles / 64);
+    };
+    arrived(step - 1, false);
+    arrived(step, true);
+  }
 }
 
 template <int LOGN, int LEV, int PRIMES>

@@ -65,6 +65,12 @@ struct BrArgs {
   uint32_t n, level, base_log, msg_bits, batch, num_luts;
   uint32_t primes;          // kPrimes (bsk, tw, cc over the 28-bit set) or kPrimes31
   uint32_t pairs;           // three primes: the CTA's shared memory holds the paired exchange buffer
+#ifdef ROSETTA_DEBUG
+  // small-batch kernel: the step (counted from 1; 0: none) whose partial products a
+  // CTA keeps back, and the waits' limit in its place (0: kWaitCycles)
+  uint32_t lose_step;
+  long long wait_cycles;
+#endif
   uint2 tw_lo[kPrimes][kTwLo];  // each prime's first twiddles again, for the constant bank
   CrtConsts cc;
 };

@@ -983,6 +983,33 @@ int rosetta_selftest_bounds(rosetta_ctx *c, void *stream) {
 #endif
 }
 
+int rosetta_selftest_lost_words(rosetta_ctx *c, uint32_t limit_us, void *stream) {
+  if (!c || limit_us == 0 || limit_us > 1000000) return ROSETTA_ERR_INVALID_ARG;
+#ifndef ROSETTA_DEBUG
+  (void)stream;
+  return ROSETTA_ERR_UNSUPPORTED_PARAMS;
+#else
+  if (!c->br_small) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
+  if (!c->have_bsk) return ROSETTA_ERR_KEYS_MISSING;
+  if (cudaSetDevice(c->device) != cudaSuccess) return ROSETTA_ERR_CUDA;
+  const cudaStream_t s = as_stream(stream);
+  int r = ensure_stage(c, 1, s);
+  if (r == ROSETTA_OK) r = ensure_big(c, 1, s);
+  if (r != ROSETTA_OK) return r;
+  // every mask word 2^63 (a~ = N): every step runs
+  const std::vector<uint64_t> lwe(lwe_words(c), 1ull << 63);
+  cudaError_t e = cudaMemcpyAsync(c->d_in, lwe.data(), lwe.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_lut, 0, sizeof(uint64_t) << c->prm.msg_bits, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // `lwe` goes out of scope
+  if (e != cudaSuccess) return cuda_fail(e);
+  BrArgs a = br_args(c, c->d_in, 1, c->d_lut, c->d_big);
+  a.lose_step = (c->prm.lwe_dim + 1) / 2;
+  a.wait_cycles = static_cast<long long>(limit_us) * 2000;  // ~2 GHz
+  e = launch_blind_rotate_small(a, c->logN, s);
+  return e == cudaSuccess ? ROSETTA_OK : cuda_fail(e);
+#endif
+}
+
 void rosetta_destroy(rosetta_ctx *c) {
   if (!c) return;
   cudaSetDevice(c->device);

@@ -422,7 +422,7 @@ template <int LOGN, bool DIG16, int LEV>
 static cudaError_t launch_br_t(const BrArgs &a, cudaStream_t s) {
   auto kern = blind_rotate_kernel<LOGN, DIG16, LEV>;
   const size_t smem = br_smem_bytes(LOGN, a.level, a.n, DIG16);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;

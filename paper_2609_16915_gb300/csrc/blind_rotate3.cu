@@ -419,7 +419,7 @@ template <int LOGN, int LEV, bool PAIRS>
 static cudaError_t launch_br3_t(const BrArgs &a, cudaStream_t s) {
   auto kern = blind_rotate3_kernel<LOGN, LEV, PAIRS>;
   const size_t smem = br3_smem_bytes(LOGN, LEV, a.n, PAIRS);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;

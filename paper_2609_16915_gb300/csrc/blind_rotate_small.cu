@@ -388,7 +388,7 @@ template <int LOGN, int LEV, int PRIMES>
 static cudaError_t launch_brs_t(const BrArgs &a, cudaStream_t s) {
   auto kern = blind_rotate_small_kernel<LOGN, LEV, PRIMES>;
   const size_t smem = brs_smem(size_t(1) << LOGN, LEV == 1, a.n, PRIMES);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
@@ -601,7 +601,7 @@ template <int LEV>
 static cudaError_t launch_brt_t(const BrArgs &a, cudaStream_t s) {
   auto kern = blind_rotate_tiny_kernel<LEV>;
   const size_t smem = br_tiny_smem_bytes(a.n);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;

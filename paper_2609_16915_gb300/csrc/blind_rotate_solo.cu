@@ -293,8 +293,7 @@ size_t br_solo_smem_bytes(uint32_t n, uint32_t workers) { return solo_table_byte
 cudaError_t launch_blind_rotate_solo(const BrArgs &a, uint32_t workers, cudaStream_t s) {
   if (workers < 1 || workers > kWorkers) return cudaErrorInvalidValue;
   const size_t smem = br_solo_smem_bytes(a.n, workers);
-  cudaError_t e = cudaFuncSetAttribute(blind_rotate_solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(blind_rotate_solo_kernel);
   if (e != cudaSuccess) return e;
   blind_rotate_solo_kernel<<<(a.batch + workers - 1) / workers, workers * kT, smem, s>>>(a);
   return cudaGetLastError();

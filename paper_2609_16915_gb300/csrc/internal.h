@@ -117,6 +117,18 @@ struct PlainMulArgs {
   CrtConsts cc;
 };
 
+// Let a kernel without static shared memory be launched with as much dynamic shared
+// memory as the device has for a block.  The limit belongs to the kernel in the whole
+// process: were it set to what each launch needs, a thread with another context (or
+// another number of workers) could lower it between this thread's call and its launch.
+template <typename K>
+inline cudaError_t allow_dynamic_smem(K kern) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return e == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most) : e;
+}
+
 // Cluster placement of a blind-rotation launch of `ctas` CTAs: packed onto
 // the SMs with room (load-balancing) once the launch fills every CTA slot of
 // the GPU at least once, spread over the SMs below that.  Measured on GB300:

@@ -113,8 +113,7 @@ __global__ void __launch_bounds__(KS_THREADS) keyswitch_kernel(const KsArgs a) {
 
 cudaError_t launch_keyswitch(const KsArgs &a, cudaStream_t s) {
   const size_t smem = static_cast<size_t>(KS_KI) * a.level * (KS_BN * sizeof(uint64_t) + KS_BM * sizeof(uint32_t));
-  cudaError_t e =
-      cudaFuncSetAttribute(keyswitch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(keyswitch_kernel);
   if (e != cudaSuccess) return e;
   dim3 grid((a.n + 1 + KS_BN - 1) / KS_BN, (a.batch + KS_BM - 1) / KS_BM, 1);
   // enough CTAs to keep every SM streaming key words: split the input words

@@ -230,7 +230,7 @@ template <int LOGN, bool DIG16>
 static cudaError_t launch_trace_t(const TraceArgs &a, cudaStream_t s) {
   auto kern = trace_kernel<LOGN, DIG16>;
   const size_t smem = trace_smem_bytes(LOGN, a.level, a.base_log);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;

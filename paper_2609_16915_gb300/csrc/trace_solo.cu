@@ -214,7 +214,7 @@ cudaError_t launch_trace_solo(const TraceArgs &a, uint32_t workers, cudaStream_t
   if (workers < 1 || workers > kTrWorkers) return cudaErrorInvalidValue;
   const size_t smem = tr_smem_bytes(workers);
   const auto kern = a.level == 2 ? trace_solo_kernel<1> : trace_solo_kernel<2>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   kern<<<(a.batch + workers - 1) / workers, workers * kTrT, smem, s>>>(a);
   return cudaGetLastError();

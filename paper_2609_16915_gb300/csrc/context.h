@@ -42,6 +42,7 @@ struct rosetta_ctx {
   uint32_t ks_limbs = 0;
   bool ks_fp8 = false;            // the limb and digit tiles are those of the 8-bit kernel
   uint64_t *d_ks_a = nullptr;     // digit tiles (scratch), as 64-bit words
+  uint64_t *d_ks_few = nullptr;   // those of the 8-bit kernel's batches up to 255, from the key's upload on
   size_t ks_a_cap = 0;
   bool have_bsk = false, have_ksk = false;
   // scratch and staging, sized in ciphertexts

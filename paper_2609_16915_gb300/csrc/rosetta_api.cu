@@ -200,8 +200,10 @@ BrArgs br_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, const u
 
 // Batches from this size on take the bf16 tensor-core key switch (where the
 // 8-bit one is not exact but this one is); smaller ones the split-K CUDA-core
-// kernel.  The 8-bit kernel takes every batch; digit scratch for batches below
-// this size is allocated with the key, so that their calls allocate nothing.
+// kernel.  The 8-bit kernel takes every batch; batches below this size have digit
+// scratch of their own, allocated with the key and kept as long as the context: their
+// calls allocate nothing, and a graph that holds one stays valid when a larger batch
+// makes the other scratch grow (and frees what it was).
 constexpr uint32_t kKsTcMinBatch = 256;
 
 KsArgs ks_args(const rosetta_ctx *c, const uint64_t *big, uint32_t batch, uint64_t *out);
@@ -211,9 +213,10 @@ cudaError_t run_keyswitch(rosetta_ctx *c, const uint64_t *big, uint32_t batch, u
   const uint32_t kN = p.glwe_dim * p.poly_size;
   if (c->d_ks_b && (c->ks_fp8 || batch >= kKsTcMinBatch)) {
     const size_t bytes = c->ks_fp8 ? ks8_a_bytes(batch, kN, p.ks_level) : 2 * ks_tc_a_words16(batch, kN, p.ks_level);
-    if (ensure(&c->d_ks_a, &c->ks_a_cap, (bytes + 7) / 8, s) != ROSETTA_OK) return cudaErrorMemoryAllocation;
+    const bool few = c->ks_fp8 && batch < kKsTcMinBatch;
+    if (!few && ensure(&c->d_ks_a, &c->ks_a_cap, (bytes + 7) / 8, s) != ROSETTA_OK) return cudaErrorMemoryAllocation;
     KsTcArgs a{};
-    a.a_tiles = reinterpret_cast<const uint16_t *>(c->d_ks_a);
+    a.a_tiles = reinterpret_cast<const uint16_t *>(few ? c->d_ks_few : c->d_ks_a);
     a.b_tiles = c->d_ks_b;
     a.big = big;
     a.out = out;
@@ -574,9 +577,7 @@ int rosetta_upload_ksk(rosetta_ctx *c, const uint64_t *ksk, size_t n_words, int 
     if (!c->d_ks_b) e = cudaMalloc(&c->d_ks_b, ks8_b_bytes(kN, p.ks_level, p.lwe_dim));
     if (e == cudaSuccess)
       e = launch_ks8_limbs(c->d_ksk, reinterpret_cast<uint8_t *>(c->d_ks_b), kN, p.ks_level, p.lwe_dim, s);
-    if (e == cudaSuccess && ensure(&c->d_ks_a, &c->ks_a_cap, ks8_a_bytes(kKsTcMinBatch - 1, kN, p.ks_level) / 8, s) !=
-                                ROSETTA_OK)
-      e = cudaErrorMemoryAllocation;
+    if (e == cudaSuccess && !c->d_ks_few) e = cudaMalloc(&c->d_ks_few, ks8_a_bytes(kKsTcMinBatch - 1, kN, p.ks_level));
     if (e != cudaSuccess) return cuda_fail(e);
   } else if (c->ks_limbs) {
     if (!c->d_ks_b) e = cudaMalloc(&c->d_ks_b, ks_tc_b_words16(kN, p.ks_level, p.lwe_dim, c->ks_limbs) * 2);
@@ -1024,6 +1025,7 @@ void rosetta_destroy(rosetta_ctx *c) {
   cudaFree(c->d_corr);
   cudaFree(c->d_ks_b);
   cudaFree(c->d_ks_a);
+  cudaFree(c->d_ks_few);
   cudaFree(c->d_big);
   cudaFree(c->d_in);
   cudaFree(c->d_out);

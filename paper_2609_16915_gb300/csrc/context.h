@@ -69,6 +69,7 @@ struct rosetta_ctx {
   bool have_lk = false;
   uint64_t *d_lk_t = nullptr, *d_lk_u = nullptr, *d_lk_R = nullptr;  // [batch][2][N] each
   size_t lk_t_cap = 0, lk_u_cap = 0, lk_R_cap = 0;
+  bool lk_short = false;          // memory was too short for several segments' scratch
   uint64_t *d_lk_I = nullptr;     // interval-index LWEs [batch][n+1]
   size_t lk_I_cap = 0;
 };

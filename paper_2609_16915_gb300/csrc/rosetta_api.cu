@@ -130,6 +130,39 @@ int ensure_stage(rosetta_ctx *c, uint32_t batch, cudaStream_t s) {
   return st == ROSETTA_OK ? ensure(&c->d_out, &c->out_words_cap, need, s) : st;
 }
 
+// Scratch of a lookup of `batch` ciphertexts: for several segments' products and
+// rotations at a time, up to 4096 ciphertexts, or where memory is too short for that for
+// one segment's.  The size for several does not fall as the batch grows, so no call
+// replaces what a larger one (or a graph that holds it) works in; and where one segment's
+// fits what is there, nothing is allocated while a graph is captured, nor after memory
+// was too short (until the next table).
+int lookup_scratch(rosetta_ctx *c, uint32_t batch, cudaStream_t s) {
+  const size_t gw = 2 * (size_t)c->prm.poly_size, one = batch * gw;
+  size_t several = std::min<size_t>((size_t)c->lk_nseg * batch, std::max(4096u, batch)) * gw;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+  const size_t have = std::min(c->lk_t_cap, c->lk_u_cap);
+  if ((c->lk_short || capture == cudaStreamCaptureStatusActive) && have >= one) several = have;
+  const auto take = [&](size_t words) {
+    int st = ensure(&c->d_lk_t, &c->lk_t_cap, words, s);
+    if (st == ROSETTA_OK) st = ensure(&c->d_lk_u, &c->lk_u_cap, words, s);
+    if (st == ROSETTA_OK) st = ensure(&c->d_lk_R, &c->lk_R_cap, one, s);
+    if (st == ROSETTA_OK) st = ensure(&c->d_lk_I, &c->lk_I_cap, batch * lwe_words(c), s);
+    return st == ROSETTA_OK ? ensure_big(c, batch, s) : st;
+  };
+  int st = take(several);
+  if (st == ROSETTA_ERR_OOM && several > one) {
+    cudaGetLastError();
+    c->lk_short = true;
+    if (c->d_lk_t) cudaFreeAsync(c->d_lk_t, s);
+    if (c->d_lk_u) cudaFreeAsync(c->d_lk_u, s);
+    c->d_lk_t = c->d_lk_u = nullptr;
+    c->lk_t_cap = c->lk_u_cap = 0;
+    st = take(one);
+  }
+  return st;
+}
+
 cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 
 // Shared front half of the entry points that take ciphertexts in and out:
@@ -850,6 +883,7 @@ int rosetta_upload_lookup_table(rosetta_ctx *c, uint32_t n_seg, const int64_t *p
   cudaFree(d_raw);
   if (e != cudaSuccess) return cuda_fail(e);
   c->lk_nseg = n_seg;
+  c->lk_short = false;
   c->have_lk = true;
   return ROSETTA_OK;
 }
@@ -871,28 +905,12 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *c, const uint64_t *glwe_x, const
   // Segments whose rotations (all by [[I]]), traces and products share one launch:
   // up to 4096 ciphertexts at a time.  A small batch is bound by the latency of a
   // rotation, a larger one loses to partly filled waves.
-  const uint32_t nseg = c->lk_nseg;
-  // (Where memory is too short for a group's scratch, one segment at a time.)
   // Measured, N = 2048, 4 segments: 256 lookups 82.3 -> 74.5 ms.
-  uint32_t group = std::min(nseg, std::max(1u, 4096u / batch));
-  const auto scratch = [&](size_t segments) {
-    int st = ensure(&c->d_lk_t, &c->lk_t_cap, segments * batch * gw, s);
-    if (st == ROSETTA_OK) st = ensure(&c->d_lk_u, &c->lk_u_cap, segments * batch * gw, s);
-    if (st == ROSETTA_OK) st = ensure(&c->d_lk_R, &c->lk_R_cap, batch * gw, s);
-    if (st == ROSETTA_OK) st = ensure(&c->d_lk_I, &c->lk_I_cap, batch * lwe_words(c), s);
-    return st == ROSETTA_OK ? ensure_big(c, batch, s) : st;
-  };
-  int r = scratch(group);
-  if (r == ROSETTA_ERR_OOM && group > 1) {
-    cudaGetLastError();
-    group = 1;
-    if (c->d_lk_t) cudaFreeAsync(c->d_lk_t, s);
-    if (c->d_lk_u) cudaFreeAsync(c->d_lk_u, s);
-    c->d_lk_t = c->d_lk_u = nullptr;
-    c->lk_t_cap = c->lk_u_cap = 0;
-    r = scratch(1);
-  }
+  const uint32_t nseg = c->lk_nseg;
+  int r = lookup_scratch(c, batch, s);
   if (r != ROSETTA_OK) return r;
+  const uint32_t group = static_cast<uint32_t>(std::min<size_t>(
+      std::min(nseg, std::max(1u, 4096u / batch)), std::min(c->lk_t_cap, c->lk_u_cap) / (batch * gw)));
   const size_t key_words = (size_t)kPrimes * gw;
   const uint32_t *kP = c->d_lk_key, *kBox = c->d_lk_key + (1 + nseg) * key_words;
   uint64_t *T = c->d_lk_t, *U = c->d_lk_u, *R = c->d_lk_R, *I = c->d_lk_I;

@@ -408,7 +408,7 @@ static cudaError_t launch_brs_t(const BrArgs &a, cudaStream_t s) {
 }
 
 size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes) {
-  return brs_smem(size_t(1) << logN, level == 1 && logN >= 11, n, primes);
+  return brs_smem(size_t(1) << logN, level == 1, n, primes);
 }
 
 // ---------------------------------------------------------------------------- the smallest ring
@@ -422,6 +422,9 @@ size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t p
 // up to two ciphertexts per SM, by the integer multiplies and the barriers beyond.
 // Measured with the key switch, n = 64, level 2, against the four-CTA cluster kernel:
 // 152 ciphertexts 172 us (312), 304: 273 (527), 2000: 1.61 ms (1.97), 20000: 14.8 (18.4).
+// One level is one row per component, transformed by itself (a pair with an empty row was
+// 8 % behind the cluster kernel from 600 ciphertexts on): 152: 117 us (158 in pairs, 230 the
+// cluster kernel), 608: 352 (494, 449), 2000: 1.15 ms (1.63, 1.49).
 // Three CTAs per SM (85 registers): 1.64 / 14.98 ms; four (64, spilling): 1.68 / 15.15.  The
 // same at N = 512 (two warps per group, six levels, n = 64): 600 us against 515 at 100
 // ciphertexts, 7.98 ms against 7.14 at 2000: not built there.
@@ -449,8 +452,12 @@ __global__ void __launch_bounds__(BrtShape::THREADS, 2)
   const uint32_t tau = threadIdx.x % T, q = group / 2, comp = group % 2;
   const uint32_t ct = blockIdx.x;
   if (!dbg_ok(ct < a.batch, a.err_flag)) return;
-  const GroupThreads pairs{group + 1u, T};
+  constexpr int NP = LEV == 1 ? 1 : 2;  // rows transformed together
+  using Rows = typename std::conditional<NP == 2, GroupThreads, GroupSingles>::type;
   const GroupSingles singles{group + 1u, T};
+  Rows row_threads;
+  row_threads.id = group + 1u;
+  row_threads.threads = T;
 
   extern __shared__ __align__(16) unsigned char smem[];
   uint2 *tw_s = reinterpret_cast<uint2 *>(smem);
@@ -509,7 +516,7 @@ __global__ void __launch_bounds__(BrtShape::THREADS, 2)
   const auto key_ok = [&](uint32_t i) {
     return dbg_ok(a.bsk_words == 0 || (static_cast<size_t>(i) * kPrimes + q + 1) * kblk <= a.bsk_words, a.err_flag);
   };
-  RowKeys<2> key;  // of the first rows of the coming step
+  RowKeys<NP> key;  // of the first rows of the coming step
   const auto load_first = [&](uint32_t i) {
     key.load(key_own + step_off(i), key_oth + step_off(i), 2 * N, key_ok(i), level);
   };
@@ -535,23 +542,23 @@ __global__ void __launch_bounds__(BrtShape::THREADS, 2)
     // ---- forward transforms, products with both components of the key ----
     uint32_t own[E], oth[E];
 #pragma unroll
-    for (uint32_t lev = 0; lev < level; lev += 2) {
+    for (uint32_t lev = 0; lev < level; lev += NP) {
       if (lev > 0)
         key.load(key_own + step_off(i) + lev * 2 * N, key_oth + step_off(i) + lev * 2 * N, 2 * N, key_ok(i),
                  level - lev);
-      uint32_t x[2][E];
+      uint32_t x[NP][E];
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < NP; ++r)
 #pragma unroll
         for (int e = 0; e < E; ++e)
           x[r][e] = lev + r < level ? biased_digit(w[e], a.base_log, lev + r) + dig_bias : p;
-      ntt_forward<LOGN, E, 2, 2>(x, tw, xb, tau, npr, pairs);
+      ntt_forward<LOGN, E, NP, NP>(x, tw, xb, tau, npr, row_threads);
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < NP; ++r)
 #pragma unroll
         for (int e = 0; e < E; ++e) x[r][e] = cond_sub(x[r][e], npr.p8);
-      mac<false, 2>(oth, x, key, 1, lev == 0, p, p_inv);
-      mac<false, 2>(own, x, key, 0, lev == 0, p, p_inv);
+      mac<false, NP>(oth, x, key, 1, lev == 0, p, p_inv);
+      mac<false, NP>(own, x, key, 0, lev == 0, p, p_inv);
     }
     if (next < a.n) load_first(next);
     part[(group ^ 1u) * 2 * T + tau] = make_uint4(oth[0], oth[1], oth[2], oth[3]);
@@ -610,7 +617,7 @@ static cudaError_t launch_brt_t(const BrArgs &a, cudaStream_t s) {
 }
 
 cudaError_t launch_blind_rotate_tiny(const BrArgs &a, cudaStream_t s) {
-  return a.level == 2 ? launch_brt_t<2>(a, s) : launch_brt_t<0>(a, s);
+  return a.level == 1 ? launch_brt_t<1>(a, s) : a.level == 2 ? launch_brt_t<2>(a, s) : launch_brt_t<0>(a, s);
 }
 
 bool br_small_supported(uint32_t logN, uint32_t level, uint32_t primes) {
@@ -628,9 +635,11 @@ cudaError_t launch_blind_rotate_small(const BrArgs &a, uint32_t logN, cudaStream
     }
   }
   switch (logN) {
-    case 8: return a.level == 2 ? launch_brs_t<8, 2, 4>(a, s) : launch_brs_t<8, 0, 4>(a, s);
-    case 9: return launch_brs_t<9, 0, 4>(a, s);
-    case 10: return launch_brs_t<10, 0, 4>(a, s);
+    case 8: return a.level == 1   ? launch_brs_t<8, 1, 4>(a, s)
+                   : a.level == 2 ? launch_brs_t<8, 2, 4>(a, s)
+                                  : launch_brs_t<8, 0, 4>(a, s);
+    case 9: return a.level == 1 ? launch_brs_t<9, 1, 4>(a, s) : launch_brs_t<9, 0, 4>(a, s);
+    case 10: return a.level == 1 ? launch_brs_t<10, 1, 4>(a, s) : launch_brs_t<10, 0, 4>(a, s);
     default: return a.level == 1 ? launch_brs_t<11, 1, 4>(a, s) : launch_brs_t<11, 2, 4>(a, s);
   }
 }

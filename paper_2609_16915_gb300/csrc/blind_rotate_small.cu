@@ -385,26 +385,45 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
 }
 
 template <int LOGN, int LEV, int PRIMES>
-static cudaError_t launch_brs_t(const BrArgs &a, cudaStream_t s) {
-  auto kern = blind_rotate_small_kernel<LOGN, LEV, PRIMES>;
-  const size_t smem = brs_smem(size_t(1) << LOGN, LEV == 1, a.n, PRIMES);
-  cudaError_t e = allow_dynamic_smem(kern);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * PRIMES * a.batch, 1, 1);
-  cfg.blockDim = dim3(BrsShape<LOGN, LEV>::T, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2 * PRIMES;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
+struct BrsKernel {
+  static constexpr auto kernel = blind_rotate_small_kernel<LOGN, LEV, PRIMES>;
+
+  // configuration of a launch of `batch` clusters (attr: room for one)
+  static cudaError_t config(uint32_t n, uint32_t batch, cudaLaunchAttribute *attr, cudaLaunchConfig_t *cfg) {
+    cudaError_t e = allow_dynamic_smem(kernel);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    *cfg = {};
+    cfg->gridDim = dim3(2 * PRIMES * batch, 1, 1);
+    cfg->blockDim = dim3(BrsShape<LOGN, LEV>::T, 1, 1);
+    cfg->dynamicSmemBytes = brs_smem(size_t(1) << LOGN, LEV == 1, n, PRIMES);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2 * PRIMES;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    return e;
+  }
+};
+
+// f(BrsKernel) of the kernel for a parameter set that br_small_supported accepts
+template <typename F>
+static cudaError_t with_brs_kernel(uint32_t logN, uint32_t level, uint32_t primes, F f) {
+  if (!br_small_supported(logN, level, primes)) return cudaErrorInvalidValue;
+  if (primes == kPrimes31) {
+    switch (level) {
+      case 1: return f(BrsKernel<12, 1, 3>());
+      case 2: return f(BrsKernel<12, 2, 3>());
+      default: return f(BrsKernel<12, 3, 3>());
+    }
+  }
+  switch (logN) {
+    case 8: return level == 1 ? f(BrsKernel<8, 1, 4>()) : level == 2 ? f(BrsKernel<8, 2, 4>()) : f(BrsKernel<8, 0, 4>());
+    case 9: return level == 1 ? f(BrsKernel<9, 1, 4>()) : f(BrsKernel<9, 0, 4>());
+    case 10: return level == 1 ? f(BrsKernel<10, 1, 4>()) : f(BrsKernel<10, 0, 4>());
+    default: return level == 1 ? f(BrsKernel<11, 1, 4>()) : f(BrsKernel<11, 2, 4>());
+  }
 }
 
 size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes) {
@@ -626,22 +645,24 @@ bool br_small_supported(uint32_t logN, uint32_t level, uint32_t primes) {
 }
 
 cudaError_t launch_blind_rotate_small(const BrArgs &a, uint32_t logN, cudaStream_t s) {
-  if (!br_small_supported(logN, a.level, a.primes)) return cudaErrorInvalidValue;
-  if (a.primes == kPrimes31) {
-    switch (a.level) {
-      case 1: return launch_brs_t<12, 1, 3>(a, s);
-      case 2: return launch_brs_t<12, 2, 3>(a, s);
-      default: return launch_brs_t<12, 3, 3>(a, s);
-    }
-  }
-  switch (logN) {
-    case 8: return a.level == 1   ? launch_brs_t<8, 1, 4>(a, s)
-                   : a.level == 2 ? launch_brs_t<8, 2, 4>(a, s)
-                                  : launch_brs_t<8, 0, 4>(a, s);
-    case 9: return a.level == 1 ? launch_brs_t<9, 1, 4>(a, s) : launch_brs_t<9, 0, 4>(a, s);
-    case 10: return a.level == 1 ? launch_brs_t<10, 1, 4>(a, s) : launch_brs_t<10, 0, 4>(a, s);
-    default: return a.level == 1 ? launch_brs_t<11, 1, 4>(a, s) : launch_brs_t<11, 2, 4>(a, s);
-  }
+  return with_brs_kernel(logN, a.level, a.primes, [&](auto k) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg;
+    const cudaError_t e = k.config(a.n, a.batch, attr, &cfg);
+    return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, k.kernel, a) : e;
+  });
+}
+
+uint32_t br_small_resident(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes) {
+  int clusters = 0;
+  const cudaError_t st = with_brs_kernel(logN, level, primes, [&](auto k) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg;
+    const cudaError_t e = k.config(n, 1, attr, &cfg);
+    return e == cudaSuccess ? cudaOccupancyMaxActiveClusters(&clusters, k.kernel, &cfg) : e;
+  });
+  if (st != cudaSuccess) cudaGetLastError();
+  return st == cudaSuccess && clusters > 0 ? static_cast<uint32_t>(clusters) : 0;
 }
 
 }  // namespace rosetta

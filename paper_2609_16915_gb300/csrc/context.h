@@ -21,6 +21,7 @@ struct rosetta_ctx {
   // external-product bound allows, the three 31-bit primes (d_tw31, cc31)
   uint32_t br_primes = rosetta::kPrimes;
   bool br_small = false;          // the small-batch kernel is compiled for the set and fits
+  uint32_t br_small_most = 0;     // largest batch it takes
   bool br3_pairs = false;         // three primes: paired exchange buffer (fits as densely)
   uint2 tw_lo[rosetta::kPrimes][rosetta::kTwLo] = {};     // first twiddles of the 28-bit set
   uint2 tw_lo31[rosetta::kPrimes31][rosetta::kTwLo] = {};  // and of the 31-bit set

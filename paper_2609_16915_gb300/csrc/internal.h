@@ -166,6 +166,7 @@ cudaError_t launch_blind_rotate_solo(const BrArgs &a, uint32_t workers, cudaStre
 // small batches (blind_rotate_small.cu): two CTAs per prime, one per component
 bool br_small_supported(uint32_t logN, uint32_t level, uint32_t primes);
 size_t br_small_smem_bytes(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes);
+uint32_t br_small_resident(uint32_t logN, uint32_t level, uint32_t n, uint32_t primes);  // clusters the GPU holds
 size_t br_tiny_smem_bytes(uint32_t n);  // N = 256, four primes: one CTA per ciphertext, any level
 cudaError_t launch_blind_rotate_tiny(const BrArgs &a, cudaStream_t s);
 cudaError_t launch_blind_rotate_small(const BrArgs &a, uint32_t logN, cudaStream_t s);

@@ -373,18 +373,26 @@ BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) 
 
 // Largest batch of the small-batch kernel: while its clusters find an SM for each
 // CTA (at N = 2048 15 clusters of 8 in GPCs of 18-20 SMs, at N = 4096 23 of 6), and
-// at the smaller rings while its CTAs of one or two warps do not crowd the SMs.
-// Measured against the cluster kernels as they were then: N = 2048, n = 742: 1
-// ciphertext 2.54 ms against 3.78, 15: 2.57 / 3.50, 16: 4.14 / 3.50; N = 4096, n = 840: 1: 6.3 / 10.7,
-// 22: 6.0 / 9.8, 24: 12.0 / 9.8; N = 512, n = 64: 8: 283 us / 578, 100: 550 / 750, 200: 1064 / 980.
-// N = 256, n = 64, against its kernel of one CTA per ciphertext, with the key
-// switch: 16: 135 us / 166, 64: 142 / 170, 76: 175 / 170 (a second cluster on an SM's
-// slots), 152: 312 / 173.
+// at the smaller rings while its CTAs of one or two warps do not crowd the SMs; never
+// more than the GPU holds at once, which for large n (the switched mask is in every CTA)
+// is the smaller number.  Measured, this kernel against the cluster kernels:
+//   N = 2048, l = 1, n = 742: 15 ciphertexts 2.41 ms, 3.12 for 16; l = 2, n = 200: 0.78 / 1.18
+//   N = 4096, l = 1, n = 150: 22: 0.85 / 1.20 (23); l = 2: 1.07 / 1.68; l = 3, n = 100: 0.87 / 1.48
+//   N = 1024, n = 200: 30: 0.68 / 0.92 (31) with two levels, 1.23 / 1.82 with five
+//   N = 1024, l = 1, n = 64: 30: 191 us / 223 (31)
+//   N = 512, n = 64: 110 (six CTAs on every SM that a cluster of 8 can use): 505 us / 712 (111) with
+//   six levels, 214 / 233 (115) with one; 112: 676 and 258
+//   N = 512, l = 1, n = 16000, where the GPU holds 51: 51: 34.1 ms / 48.9 (52); 60: 64.5 / 48.7
+// N = 256, n = 64, against its kernel of one CTA per ciphertext: 66: 130 us / 156 with two
+// levels, 113 / 116 with one.
 static uint32_t br_small_max(const rosetta_ctx *c) {
-  const uint32_t S = c->sms;
-  if (c->br_primes == kPrimes31) return c->logN == 12 ? S * 3 / 20 : 0;
-  if (c->logN == 8) return S * 7 / 16;
-  return c->logN == 9 ? S * 3 / 4 : c->logN == 10 ? S / 5 : S / 10;
+  const uint32_t S = c->sms, resident = br_small_resident(c->logN, c->prm.pbs_level, c->prm.lwe_dim, c->br_primes);
+  uint32_t most = S / 10;
+  if (c->br_primes == kPrimes31)
+    most = c->logN == 12 ? S * 3 / 20 : 0;
+  else if (c->logN <= 10)
+    most = c->logN == 8 ? S * 7 / 16 : c->logN == 9 ? S * 8 / 11 : S / 5;
+  return std::min(most, resident);
 }
 
 // Blind rotation of a batch: the small-batch kernel, the cluster kernels (at N = 256
@@ -399,7 +407,7 @@ static uint32_t br_small_max(const rosetta_ctx *c) {
 // is still ahead: r <= 3/4 S and S < r <= 5/4 S.
 cudaError_t run_blind_rotate(const rosetta_ctx *c, const BrArgs &a, cudaStream_t s) {
   const auto cluster = [&](const BrArgs &b) {
-    if (c->br_small && b.batch <= br_small_max(c)) return launch_blind_rotate_small(b, c->logN, s);
+    if (b.batch <= c->br_small_most) return launch_blind_rotate_small(b, c->logN, s);
     return c->logN == 8 ? launch_blind_rotate_tiny(b, s) : launch_blind_rotate(b, c->logN, c->dig16, s);
   };
   if (!c->br_qf) return cluster(a);
@@ -488,6 +496,7 @@ int rosetta_params_init(rosetta_ctx **out, const rosetta_params *p, int cuda_dev
   }
   c->br_small = br_small_supported(logN, p->pbs_level, c->br_primes) &&
                 br_small_smem_bytes(logN, p->pbs_level, p->lwe_dim, c->br_primes) <= (size_t)max_smem;
+  if (c->br_small) c->br_small_most = br_small_max(c);
   for (int q = 0; q < kPrimes; ++q)
     for (int m = 0; m < kTwLo; ++m) {
       c->tw_lo[q][m] = tw[((size_t)q << logN) + m];

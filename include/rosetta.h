@@ -158,7 +158,7 @@ int rosetta_blind_rotate_extract_batch(rosetta_ctx *ctx, const uint64_t *lwe_in,
  * product runs on the tensor cores: at every batch size with 13 limbs of 5
  * bits per key word in e4m3 (beta_ks <= 5 and 2^(beta_ks-1) 16 kN l_ks < 2^24),
  * with a digit scratch of batch (kN l_ks) bytes owned by the context (for up to
- * 255 ciphertexts allocated with the key); else from 256 ciphertexts on with 8
+ * 255 ciphertexts one of its own, kept from the key's upload on); else from 256 ciphertexts on with 8
  * or 16 limbs in bf16 (beta_ks <= 8 and
  * 2^(beta_ks-1) (2^(64/limbs)-1) kN l_ks < 2^24); else on the CUDA cores.  The
  * words are the same either way.  A bounded wait inside a tensor-core kernel
@@ -203,11 +203,12 @@ int rosetta_blind_rotate_glwe_batch(rosetta_ctx *ctx, const uint64_t *lwe_in, ui
  * `level` GLWE encryptions under S of sigma_k(S) * 2^(64 - lev*base_log).
  * Raw layout [log2 N][level][2][N] (n_words = log2 N * level * 2 * N);
  * level must be even, 1 <= base_log <= 28, base_log * level <= 64.  Converted
- * on the device like the BSK.  N = 8192 returns UNSUPPORTED_PARAMS: the
- * trace, plaintext-product and lookup kernels keep a whole ciphertext's
- * transform state per cluster in shared memory (about 244 KB per CTA at
- * N = 8192 against the 227 KB a CTA may have); the paper's lookups run on
- * an N_br = 2048 ring.  Errors: INVALID_ARG, UNSUPPORTED_PARAMS, CUDA, OOM. */
+ * on the device like the BSK.  Limits of the interface: N = 8192 returns
+ * UNSUPPORTED_PARAMS (the trace, plaintext-product and lookup kernels are built
+ * for N <= 4096; the paper's lookups run on an N_br = 2048 ring), and so do
+ * levels for which (26.5 + level) N bytes exceed a block's shared memory (on a
+ * 227 KB device: more than 30 at N = 4096).  Errors: INVALID_ARG, UNSUPPORTED_PARAMS,
+ * CUDA, OOM. */
 int rosetta_upload_trace_keys(rosetta_ctx *ctx, const uint64_t *keys, size_t n_words, uint32_t base_log,
                               uint32_t level, int src_is_device, void *stream);
 
@@ -268,7 +269,9 @@ int rosetta_upload_lookup_table(rosetta_ctx *ctx, uint32_t n_seg, const int64_t 
  * synchronisation.  Per ciphertext: n_seg + 2 plaintext products, n_seg + 2
  * blind rotations, one key switch, n_seg + 1 traces; the segments' products,
  * rotations and traces share launches, up to 4096 ciphertexts each, with
- * scratch for as many (2 x 2N words each).  Errors: INVALID_ARG,
+ * scratch for min(n_seg batch, max(4096, batch)) ciphertexts (2 x 2N words
+ * each); where memory is too short for it, and while a graph is captured, the
+ * groups are as large as the scratch there is.  Errors: INVALID_ARG,
  * KEYS_MISSING, CUDA, OOM. */
 int rosetta_segmented_lookup_batch(rosetta_ctx *ctx, const uint64_t *glwe_x, const uint64_t *lwe_seg, uint32_t batch,
                                    uint64_t *glwe_out, void *stream);
@@ -287,8 +290,9 @@ int rosetta_segmented_lookup_batch(rosetta_ctx *ctx, const uint64_t *glwe_x, con
  * address in the current CUDA context; the first call on a device (and the
  * first after a device reset) loads the library's device code: make it
  * before any stream capture.  The key switch is the CUDA-core kernel at
- * every batch size, because the tensor-core ones need digit tiles in
- * allocated memory (same words).  All calls on a device share the array:
+ * every batch size: the tensor-core ones' digit tiles grow with the batch, and
+ * those a context keeps for small batches are not used here (same words).  All
+ * calls on a device share the array:
  * calls whose work overlaps on the GPU race and must be serialised by the
  * caller.  Errors: INVALID_ARG, KEYS_MISSING, CUDA. */
 int rosetta_pbs_batch_noalloc(rosetta_ctx *ctx, const uint64_t *lwe_in, uint32_t batch,

@@ -21,9 +21,9 @@
 // (1 u); a sum of 2 l products adds (4 l + 2) u.  By Cauchy-Schwarz a
 // coefficient of the product is off by less than
 //   (3.9 log2 C + 1 + (4 l + 2) + 3.8 log2 C) u sum_r |d_r| |g_r|,
-// below 100 u times (k+1) l N 2^(beta-1) 2^63 for C <= 1024 and l <= 3
-// (kCfftErr; the product of three stages' second-order terms is far below the
-// slack).
+// below kCfftErr = 100 u times (k+1) l N 2^(beta-1) 2^63 for C <= 1024 and l <= 3 (the
+// trace's sums of four products are those of l = 2); the product of three stages'
+// second-order terms is far below the slack.
 #pragma once
 #include <stdint.h>
 

@@ -22,10 +22,10 @@ constexpr uint32_t kPrimeList[kPrimes] = {268369921u, 268271617u, 268238849u, 26
 constexpr int kPrimes31 = 3;
 constexpr uint32_t kPrime31List[kPrimes31] = {2147352577u, 2147205121u, 2147074049u};
 
-// The float quotient (QF): a blind rotation over the first three 28-bit primes
-// whose fourth CTA estimates the product's size X / M3 with single-precision
-// complex transforms (cfft.cuh) instead of computing a fourth residue.  The
-// estimate arrives scaled by 2^kQfShift; |X| / M3 <= 2^(kQfBits - 83.99).
+// The float quotient (QF): exact residues over the first three 28-bit primes, and in
+// place of a fourth residue an estimate of the product's size X / M3 by
+// single-precision complex transforms (cfft.cuh), which the same worker computes.  The
+// estimate is scaled by 2^kQfShift; |X| / M3 <= 2^(kQfBits - 83.99).
 constexpr int kPrimesQf = 3;
 constexpr int kQfShift = 16;
 constexpr int kQfBits = 98;
@@ -43,7 +43,7 @@ struct PrimeConsts {
 struct CrtConsts {
   PrimeConsts pr[kPrimes];
   uint64_t M_mod64;   // M mod 2^64
-  uint64_t qf_base;   // 2^(31 - kQfShift) M mod 2^64: undoes the offset of crt_quotient_qf
+  uint64_t qf_base;   // 2^(31 - kQfShift) M mod 2^64: undoes the offset of qf_quotient
 };
 
 constexpr int kTwLo = 64;  // entries of the first six stages

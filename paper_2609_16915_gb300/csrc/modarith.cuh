@@ -45,13 +45,20 @@ __device__ __forceinline__ uint32_t crt_quotient(uint32_t ysum) { return (ysum +
 // this prime set, so the estimate stays within 0.46 of the integer.
 __device__ __forceinline__ uint32_t crt_quotient31(uint32_t ysum) { return (ysum + (1u << 27)) >> 28; }
 
+// Worst case of the float transforms' estimate, in units of 2^-24 of the bound on |X|
+// (derived in cfft.cuh).
+constexpr double kCfftErr = 100.0;
+static_assert(kCfftErr / 16777216.0 * (1ull << (kQfBits / 2)) * (1ull << (kQfBits - kQfBits / 2)) <
+                  0.1 * kPrimeList[0] * kPrimeList[1] * kPrimeList[2],
+              "the estimate of X / M3 is within 0.1 of its exact value");
+
 // The quotient of three 28-bit primes where X may be many times their product
 // M3: round(sum_q y_q / p_q - X / M3), from ysum = sum_q (y_q >> 17) and est =
 // 2^kQfShift X / M3 as the float transforms give it, plus an offset of
 // 2^(31 - kQfShift) that keeps it positive.  The primes lie in (2^28 - 2^18,
 // 2^28): y / 2^28 undershoots y / p by less than 2^-7 per prime (the shift adds
 // 2^-11), the three together by less than 2^-5.  est is within
-// 100 x 2^-24 x 2^98 / 2^83.99 < 0.1 of its exact value (cfft.cuh; |X| <=
+// kCfftErr 2^-24 2^98 / 2^83.99 < 0.1 of its exact value (|X| <=
 // 2^98), so the sum stays within 0.14 of an integer and rounds to it; |est|
 // <= 2^30.02 fits the conversion.
 __device__ __forceinline__ uint32_t qf_quotient(uint32_t ysum, float est) {

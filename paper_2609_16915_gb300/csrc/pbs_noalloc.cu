@@ -27,9 +27,10 @@
 // words of every ciphertext slot it uses before the key switch reads them.
 //
 // The key switch is the CUDA-core kernel (keyswitch_kernel) at every batch
-// size: the tensor-core kernel that rosetta_pbs_batch uses from 256
-// ciphertexts on needs digit tiles in a buffer the library allocates.  Both
-// give the same words.
+// size.  The tensor-core kernels that rosetta_pbs_batch uses (for bases up to 2^5 at
+// every batch size, for wider ones from 256 ciphertexts on) need digit tiles, whose
+// buffer grows with the batch; the tiles that a context keeps for up to 255
+// ciphertexts are not used here.  All give the same words.
 #include <cuda_runtime.h>
 
 #include "context.h"

@@ -330,6 +330,8 @@ TraceArgs trace_args(const rosetta_ctx *c, const uint64_t *in, uint32_t batch, u
 // cluster kernel about 42 us + 1.24 a ciphertext (152: 226, 228: 323, 304: 419, 456:
 // 603).  So whole waves of 3 S go to three workers, and of the rest r those up to
 // 5/3 S and from 2 S to 9/4 S to clusters, up to 2 S to two workers, more to three.
+// The lines are those of four levels.  With two (2^24 x 2): w = 2, 3: 226, 315 us, clusters
+// 163 (152), 238 (228), 253 (253), 307 (305), 340 (342): both come up to 12 % late.
 cudaError_t run_trace(const rosetta_ctx *c, const TraceArgs &a, cudaStream_t s) {
   if (!c->trk_qf) return launch_trace(a, c->logN, s);
   const uint32_t S = c->sms, wave = 3 * S;
@@ -741,14 +743,14 @@ int rosetta_upload_trace_keys(rosetta_ctx *c, const uint64_t *keys, size_t n_wor
   if (base_log < 1 || base_log > 28 || level < 2 || (level & 1u) || base_log * level > 64)
     return ROSETTA_ERR_UNSUPPORTED_PARAMS;
   if (c->logN > 12) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
-  // exact CRT: level N 2^(base_log-1) 2^63 below M/2 > 2^114
+  // exact CRT: level N 2^(base_log-1) 2^63 <= 2^110, below M / 2 > 2^110.99
   {
     int e = 0;
     while ((1ull << e) < (uint64_t)level * p.poly_size) ++e;
     if (63 + (base_log - 1) + e + 1 > 111) return ROSETTA_ERR_UNSUPPORTED_PARAMS;
   }
-  // the documented limit on levels: 26.5 N + level N bytes per CTA (the kernel
-  // itself needs less)
+  // the interface's limit on levels, (26.5 + level) N bytes within a block's shared memory
+  // (the kernel itself needs 21 N + level N / 2, or level N above base 2^16)
   int max_smem = 0;
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
   if ((size_t)p.poly_size * (53 + 2 * (size_t)level) / 2 > (size_t)max_smem) return ROSETTA_ERR_UNSUPPORTED_PARAMS;

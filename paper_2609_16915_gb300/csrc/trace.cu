@@ -43,8 +43,8 @@ struct TrShape {
   static constexpr int E = 8;
   static constexpr int T = N / E;
   static constexpr int Q = N / 4;
-  // resident CTAs per SM the register allocation must allow (4 x 50-54 KB of
-  // shared memory at N = 2048, 2 x 100-108 KB at 4096, four levels)
+  // resident CTAs per SM the register allocation must allow (4 x 46-50 KB of
+  // shared memory at N = 2048, 2 x 92-100 KB at 4096, four levels of 16- or 32-bit digits)
   static constexpr int MIN_CTAS = LOGN == 11 ? 4 : (LOGN == 12 ? 2 : 1);
   static constexpr int XB_WORDS = 2 * (N + N / 8);  // pairs of words; the outgoing residues (2N) afterwards
 };

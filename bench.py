@@ -56,12 +56,13 @@ def min_primes(p) -> int:
     return math.ceil(bits / 31)
 
 
-def int_ops_per_pbs(p):
+def int_ops_per_pbs(p, primes=None):
     """Algorithmic 32-bit integer operations of one PBS: (blind rotation,
     key switch).  Counting convention: NTT butterflies 8 ops, pointwise
     multiply-accumulate 6, CRT 10 per prime, decomposition 6 per level,
-    rotation/accumulate 4, per coefficient; key switch 3 per digit x word."""
-    P = min_primes(p)
+    rotation/accumulate 4, per coefficient; key switch 3 per digit x word.
+    `primes`: another number of primes than the fewest of 31 bits."""
+    P = primes or min_primes(p)
     k1, l, N = p.k + 1, p.pbs_level, p.N
     per_cmux = ((k1 * l + k1) * P * (N // 2) * int(math.log2(N)) * 8 + k1 * l * k1 * P * N * 6
                 + k1 * N * 10 * P + k1 * N * l * 6 + k1 * N * 4)
@@ -127,13 +128,64 @@ def br_solo(p) -> bool:
     return p.N == 2048 and p.pbs_level == 1 and p.pbs_base_log <= 24
 
 
+SOLO, TINY = "blind_rotate_solo_kernel (3 primes and a float quotient)", "blind_rotate_tiny_kernel (4 primes)"
+
+
+def three_primes(p) -> bool:
+    """Does the context take three 31-bit primes (at the named sets' dimensions)?"""
+    return (p.N in (4096, 8192) and p.pbs_level <= 3 and p.pbs_base_log <= 16
+            and 20 * 2 * p.pbs_level * p.N << (p.pbs_base_log + 62) <= 9 * 2147352577 * 2147205121 * 2147074049)
+
+
+def br_parts(p, batch, sms):
+    """Blind-rotation kernels of one call with their ciphertexts, as
+    run_blind_rotate splits a batch (at dimensions whose small-batch clusters all
+    find room)."""
+    three = three_primes(p)
+    if p.N == 8192 or (p.N == 4096 and not three) or (p.N == 2048 and p.pbs_level > 2):
+        small = 0
+    elif p.N == 4096:
+        small = sms * 3 // 20
+    else:
+        small = {256: sms * 7 // 16, 512: sms * 8 // 11, 1024: sms // 5, 2048: sms // 10}[p.N]
+
+    def clusters(b):
+        primes = f"({3 if three else 4} primes)"
+        if b <= small:
+            return f"blind_rotate_small_kernel {primes}", b
+        return (TINY if p.N == 256 else f"blind_rotate{'3' if three else ''}_kernel {primes}"), b
+
+    if not br_solo(p):
+        return [clusters(batch)]
+    rest = batch % (3 * sms)
+    if rest > 2 * sms:
+        return [(SOLO, batch)]
+    parts = [(SOLO, batch - rest)] if batch > rest else []
+    if rest:
+        on_clusters = rest <= sms - sms // 4 or sms < rest <= sms + sms // 4
+        parts.append(clusters(rest) if on_clusters else (SOLO, rest))
+    return parts
+
+
+def kernel_name(p, batch, sms):
+    """The kernels of br_parts, with their shares where there are several."""
+    parts = br_parts(p, batch, sms)
+    names = [k for k, _ in parts]
+    if len(set(names)) == 1:
+        return names[0]
+    return " + ".join(f"{k} on {b}" for k, b in parts)
+
+
+def executed_ops(p, batch, sms) -> float:
+    """Integer operations by the same convention with the primes that run: the
+    worker kernel's three (its float transforms not counted) where the convention
+    counts four."""
+    return sum(b * int_ops_per_pbs(p, 3 if k == SOLO else None)[0] for k, b in br_parts(p, batch, sms))
+
+
 def br_launches(p, batch, sms) -> int:
-    """Blind-rotation kernels of one call: whole waves on three workers per SM
-    and the rest as run_blind_rotate splits it."""
-    full, rest = divmod(batch, 3 * sms)
-    if not br_solo(p) or rest == 0 or full == 0 or rest > 2 * sms:
-        return 1
-    return 2
+    """Blind-rotation kernels of one call."""
+    return len(br_parts(p, batch, sms))
 
 
 def trace_launches(p, batch, sms) -> int:
@@ -411,8 +463,9 @@ def run_lookup(args, p, batch, torch, dev, R, clock_sampler):
         "config": {"workload": f"segmented lookup, {n_seg} segments, ring of {describe(p, batch)}, "
                                f"trace gadget 2^{tb} x {tl}", "batch": batch,
                    "l2": "flushed between steps (256 MB write)", "keys": "uniform words, resident"},
-        "roofline": {"bound": "alu", "kernel": "blind_rotate_kernel (GLWE test polynomials)", "achieved": achieved,
-                     "peak": alu_peak, "unit": "Tops/s (int32)", "frac": achieved / alu_peak, "traffic": None,
+        "roofline": {"bound": "alu", "kernel": kernel_name(p, batch, sms) + ", GLWE test polynomials",
+                     "achieved": achieved, "peak": alu_peak, "unit": "Tops/s (int32)", "frac": achieved / alu_peak,
+                     "frac_executed": executed_ops(p, batch, sms) / (br_ops * batch) * achieved / alu_peak, "traffic": None,
                      "kernel_ms": br_ms, "trace_ms": tr_ms,
                      "path_ops_per_lookup": ops, "path_achieved": path_achieved,
                      "path_frac": path_achieved / alu_peak},
@@ -470,8 +523,9 @@ def run_multi_lut(args, p, batch, torch, dev, R, clock_sampler):
         "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
         "config": {"workload": describe(p, batch) + ", 4 LUTs round-robin", "batch": batch,
                    "l2": "flushed between steps (256 MB write)", "keys": "uniform words, resident"},
-        "roofline": {"bound": "alu", "kernel": "blind_rotate_kernel + key switch (whole step)", "achieved": achieved,
-                     "peak": alu_peak, "unit": "Tops/s (int32)", "frac": achieved / alu_peak, "traffic": None},
+        "roofline": {"bound": "alu", "kernel": kernel_name(p, batch, sms) + ", key switch (whole step)",
+                     "achieved": achieved, "peak": alu_peak, "unit": "Tops/s (int32)", "frac": achieved / alu_peak,
+                     "frac_executed": executed_ops(p, batch, sms) / (br_ops * batch) * achieved / alu_peak, "traffic": None},
         "gpu_launches": (br_launches(p, batch, sms) + (2 if ks_fp8(p) or ks_tensor_limbs(p, batch) else 1)) * args.steps,
         "clocks": clk.summary(),
     }
@@ -506,12 +560,6 @@ def butterfly_rate(rates, primes):
     rotation runs: the lazy one of the 28-bit primes (five instructions) or
     the one of the 31-bit primes (nine)."""
     return rates["butterfly_p31"]["per_clk_per_sm"] / 9.0 if primes == 3 else rates["butterfly"]["per_clk_per_sm"] / 5.0
-
-
-def kernel_name(primes, p=None):
-    if p is not None and br_solo(p):
-        return "blind_rotate_solo_kernel (3 primes and a float quotient)"
-    return "blind_rotate3_kernel (3 primes)" if primes == 3 else "blind_rotate_kernel (4 primes)"
 
 
 def measure_other_config(name, torch, dev, R, steps, warmup, sms, sm_max, rates):
@@ -560,7 +608,7 @@ def measure_other_config(name, torch, dev, R, steps, warmup, sms, sm_max, rates)
     del lwe, out, big, flush
     torch.cuda.empty_cache()
     return {"workload": describe(p, batch), "value": batch / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
-            "steps": steps, "warmup": warmup, "kernel": kernel_name(primes), "blind_rotation_ms": br_ms,
+            "steps": steps, "warmup": warmup, "kernel": kernel_name(p, batch, sms), "blind_rotation_ms": br_ms,
             "achieved_tops": achieved, "frac": achieved / (sms * 128 * sm_max * 1e6 / 1e12),
             "frac_of_butterfly_rate_peak": achieved / (bfly_per_clk * 8 * sms * sm_max * 1e6 / 1e12),
             "butterflies_per_clk_per_sm": round(bfly_per_clk, 2)}
@@ -738,8 +786,11 @@ def main():
         "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
         "config": {"workload": describe(p, batch), "batch": batch, "parallelism": f"dp{world}" if world > 1 else "none",
                    "l2": "flushed between steps (256 MB write)", "keys": "uniform words, resident"},
-        "roofline": {"bound": "alu", "kernel": kernel_name(primes, p), "achieved": achieved, "peak": alu_peak,
+        "roofline": {"bound": "alu", "kernel": kernel_name(p, batch, sms), "achieved": achieved, "peak": alu_peak,
                      "unit": "Tops/s (int32)", "frac": achieved / alu_peak, "traffic": measured_traffic(p, batch),
+                     "ops_basis": f"the convention's count, {min_primes(p)} primes of 31 bits; frac_executed: the primes "
+                                  "that run, without the worker kernel's float transforms",
+                     "frac_executed": executed_ops(p, batch, sms) / (br_ops * batch) * achieved / alu_peak,
                      "peak_basis": f"{sms} SMs x 128 int32 lanes x {sm_max:.0f} MHz (sm_max_mhz of MEASURED_PEAKS.json)",
                      "kernel_ms": br_ms, "keyswitch_ms": ks_ms, "keyswitch": ks_roof,
                      "pbs_roof": pbs_roof, "pbs_frac_of_roof": value / world / pbs_roof,

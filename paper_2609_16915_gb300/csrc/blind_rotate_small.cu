@@ -26,9 +26,9 @@
 // st.async, 2.42 with 2p and 8p loaded as values (NttPrime).
 //
 // Every wait gives up after about two seconds and raises the error flag.  The CTA
-// then finishes the step with what it has, all threads leave the loop after it
-// (no further words are sent and no mbarrier is armed again), and nothing is written
-// out.  Its peers miss its words in the next step and leave the same way, so every CTA
+// then finishes the step with what it has, all threads leave the loop after it (no
+// further words are sent; the next step's mbarriers are armed once, to count what still
+// comes), and nothing is written out.  Its peers miss its words in the next step and leave the same way, so every CTA
 // comes to the cluster barrier at the end; the CTA that gave up then waits, with a limit,
 // for the words that were still on their way to it: the rest of its last step's and, a
 // step early, those of the next.
@@ -223,6 +223,10 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
     const uint32_t at = atil[i];
     const uint32_t odd = step & 1u, phase = (step >> 1) & 1u;
     const uint32_t part_bar = bar0 + 16u * odd, res_bar = part_bar + 8u;
+    if (tau == 0) {
+      expect_tx(part_bar, N * 4u);
+      expect_tx(res_bar, (PRIMES - 1) * N * 4u);
+    }
     // A wait of the last step gave up: the same for all threads, as it was written before that
     // step's last barrier and is not again before this one's first.  (The word is needed
     // anyway; a flag of its own, or a barrier that reduces the threads', cost 1 to 3 %.)
@@ -243,10 +247,6 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
         if (a.err_flag) atomicExch(a.err_flag, 2u);
       }
     };
-    if (tau == 0) {
-      expect_tx(part_bar, N * 4u);
-      expect_tx(res_bar, (PRIMES - 1) * N * 4u);
-    }
 
     // ---- forward transforms, products with both components of the key ----
     uint32_t own[E], oth[E];
@@ -368,8 +368,9 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
   cluster.sync();  // no CTA leaves while a peer may still store into it
   if (gave_up && tau == 0) {
     // Every store has been issued by now and takes microseconds to arrive.  The next
-    // step's mbarriers are armed here to count the early words: their phase before,
-    // the last step's but one, was complete when this step was run.
+    // step's mbarriers count the early words: they were armed before the loop was left,
+    // or after the last step of all are armed here (their phase before, the last step's but
+    // one, was complete when that step was run).
     const auto arrived = [&](uint32_t st, bool arm) {
       const uint32_t pb = bar0 + 16u * (st & 1u), ph = (st >> 1) & 1u;
       if (arm) {
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(BrsShape<LOGN, LEV>::T, LOGN == 11 ? 2 : 1)
       mbar_wait_cluster(pb + 8u, ph, wait_cycles / 64);
     };
     arrived(step - 1, false);
-    arrived(step, true);
+    arrived(step, i >= a.n);
   }
 }
 

@@ -147,7 +147,7 @@ def br_parts(p, batch, sms):
     elif p.N == 4096:
         small = sms * 3 // 20
     else:
-        small = {256: sms * 7 // 16, 512: sms * 8 // 11, 1024: sms // 5, 2048: sms // 10}[p.N]
+        small = {256: sms * 7 // 16, 512: sms * 3 // 4 if p.pbs_level >= 6 else sms * 8 // 11, 1024: sms // 5, 2048: sms // 10}[p.N]
 
     def clusters(b):
         primes = f"({3 if three else 4} primes)"

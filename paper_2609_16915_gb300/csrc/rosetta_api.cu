@@ -375,15 +375,15 @@ BrArgs br_slice(const rosetta_ctx *c, BrArgs a, uint32_t first, uint32_t count) 
 
 // Largest batch of the small-batch kernel: while its clusters find an SM for each
 // CTA (at N = 2048 15 clusters of 8 in GPCs of 18-20 SMs, at N = 4096 23 of 6), and
-// at the smaller rings while its CTAs of one or two warps do not crowd the SMs; never
-// more than the GPU holds at once, which for large n (the switched mask is in every CTA)
-// is the smaller number.  Measured, this kernel against the cluster kernels:
+// at the smaller rings while its CTAs of one or two warps do not crowd the SMs; and no
+// more than the GPU holds at once where large n (the switched mask is in every CTA) makes
+// that the smaller number.  Measured, this kernel against the cluster kernels:
 //   N = 2048, l = 1, n = 742: 15 ciphertexts 2.41 ms, 3.12 for 16; l = 2, n = 200: 0.78 / 1.18
 //   N = 4096, l = 1, n = 150: 22: 0.85 / 1.20 (23); l = 2: 1.07 / 1.68; l = 3, n = 100: 0.87 / 1.48
 //   N = 1024, n = 200: 30: 0.68 / 0.92 (31) with two levels, 1.23 / 1.82 with five
 //   N = 1024, l = 1, n = 64: 30: 191 us / 223 (31)
-//   N = 512, n = 64: 110 (six CTAs on every SM that a cluster of 8 can use): 505 us / 712 (111) with
-//   six levels, 214 / 233 (115) with one; 112: 676 and 258
+//   N = 512, n = 64: 110 (six CTAs on every SM that a cluster of 8 can use): 270 us / 325 (111) with two
+//   levels, 214 / 233 with one; 112, in a second round: 364 and 258, but with six 676 / 713
 //   N = 512, l = 1, n = 16000, where the GPU holds 51: 51: 34.1 ms / 48.9 (52); 60: 64.5 / 48.7
 // N = 256, n = 64, against its kernel of one CTA per ciphertext: 66: 130 us / 156 with two
 // levels, 113 / 116 with one.
@@ -393,8 +393,10 @@ static uint32_t br_small_max(const rosetta_ctx *c) {
   if (c->br_primes == kPrimes31)
     most = c->logN == 12 ? S * 3 / 20 : 0;
   else if (c->logN <= 10)
-    most = c->logN == 8 ? S * 7 / 16 : c->logN == 9 ? S * 8 / 11 : S / 5;
-  return std::min(most, resident);
+    most = c->logN == 8    ? S * 7 / 16
+           : c->logN == 10 ? S / 5
+                           : c->prm.pbs_level >= 6 ? S * 3 / 4 : S * 8 / 11;
+  return resident < most - most / 10 ? resident : most;  // (a few clusters in a second round run beside the first's)
 }
 
 // Blind rotation of a batch: the small-batch kernel, the cluster kernels (at N = 256
